@@ -357,9 +357,10 @@ int ntu_stage_times(ntu_ctx* ctx, double* ms_out);
  * reset), into counts[8]: counts[0] ALS solves whose tolerance selection
  * (Eq. 4) was decided by Gershgorin discs (every candidate tolerance keeps
  * every eigenpair of g_A) and solved by conjugate gradients, counts[1] ALS
- * solves decided by a shifted Cholesky factorisation and solved by
- * iterative refinement, counts[2] ALS solves through the eigendecomposition
- * and the full selection, counts[3] metrics certified positive definite by
+ * solves decided by one shifted triangular factorisation (every tolerance
+ * keeps every eigenpair) and solved through factors, counts[2] ALS solves
+ * that compared tolerances (by further factorisations or through the
+ * spectrum), counts[3] metrics certified positive definite by
  * Gershgorin discs, counts[4] by Cholesky, counts[5] metrics repaired
  * through the eigendecomposition (Sec. II), counts[6] QRs of gated matrices
  * (Fig. 2(b)) by double-FP32 CholeskyQR2 (mixed contexts), counts[7] by

@@ -11,24 +11,12 @@
 
 #include <type_traits>
 
+#include "als_slow.cuh"
 #include "als_types.cuh"
 
 namespace ntu {
 
 // ---------------------------------------------------------------- ALS
-// Candidate relative tolerances 1e-k of the pseudo-inverse (Eq. 4), as
-// correctly rounded decimal literals.
-__device__ __forceinline__ double als_tau(int k) {
-  switch (k) {
-    case 0: return 1e0;   case 1: return 1e-1;  case 2: return 1e-2;  case 3: return 1e-3;
-    case 4: return 1e-4;  case 5: return 1e-5;  case 6: return 1e-6;  case 7: return 1e-7;
-    case 8: return 1e-8;  case 9: return 1e-9;  case 10: return 1e-10; case 11: return 1e-11;
-    case 12: return 1e-12; case 13: return 1e-13; case 14: return 1e-14; case 15: return 1e-15;
-    case 16: return 1e-16; case 17: return 1e-17; case 18: return 1e-18; case 19: return 1e-19;
-    default: return 1e-20;
-  }
-}
-
 // The double-FP32 split of the isometric factor (during a build) and of the
 // CG direction (during a solve) live in the SVD work array W, which only the
 // tilts use; this keeps the per-CTA footprint low enough for three CTAs per
@@ -790,6 +778,8 @@ static __device__ void als_source(AlsShared& sm, const AlsArgs& a, int side, dou
 // sigma / (lambda_min - sigma).  Both read the lower triangle of gX (tier 1
 // mirrors it into the upper one).  Returns 1 when solved, 0 when neither
 // proof holds or an iteration stalls; the caller then takes the eigen path.
+// The FP64 contexts have tier 2 in als_solve_certified and the eigen path in
+// als_solve_spectrum (als_slow.cuh).
 static __device__ void als_mirror(double2* gX, int nA);
 
 // Upper triangle of the double-FP32 copy from its lower triangle.
@@ -885,6 +875,7 @@ static __device__ void als_matvec(AlsShared& sm, const double2* A, const float4*
   __syncthreads();
 }
 
+template <bool F64>
 static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, double2* gX,
                                      double2* gC, const double2* jv, double tau_max) {
   const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31, nA = a.nA;
@@ -897,7 +888,7 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
   // reads every entry anyway (the product is dropped if tier 2 runs); that
   // rounding (< 1e-5 relative for n_A <= 256) is covered by inflating s_i by
   // 1e-4.
-  const bool df = a.df != 0;
+  const bool df = !F64 && a.df != 0;
   const float4* gXdf = reinterpret_cast<const float4*>(gC);
   const double2* M0 = side == 0 ? sm.MA : sm.MB;
   double glo = INFINITY, ghi = -INFINITY;
@@ -1012,7 +1003,20 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
     }
     __syncthreads();
   }
-  // Tier 2: a Cholesky factorisation of gX - sigma I proves the same bound.
+  if constexpr (F64) {
+    const int by = nA <= LOW_SH_MAX ? als_solve_certified<true>(sm, a, side, gX, gC, jv, bmax)
+                                    : als_solve_certified<false>(sm, a, side, gX, gC, jv, bmax);
+    if (tid == 0) {
+      if (by == 1) sm.n_fast += 1;
+      if (by == 2) sm.n_eig += 1;
+    }
+    __syncthreads();
+    return by != 0;
+  } else {
+  // Tier 2 on the mixed contexts, whose results feed roundings to FP32 and
+  // BF16 in the next bond's environment: the arithmetic of these solves is
+  // kept to the last bit.  A Cholesky factorisation of gX - sigma I proves the
+  // same bound.
   for (int idx = tid; idx < nA * nA; idx += NTU_CTA)
     if (idx % nA >= idx / nA) gC[idx] = gX[idx];
   __syncthreads();
@@ -1053,6 +1057,7 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
   if (tid == 0) { sm.tau_sel = tau_max; sm.n_fast += 1; }
   __syncthreads();
   return 1;
+  }
 }
 
 // Fill the upper triangle of gX from its lower triangle (the eigen path
@@ -1119,9 +1124,12 @@ static __device__ void als_solve(AlsShared& sm, const AlsArgs& a, int side, doub
 // spills; 3: 80 registers, for batches of more than two items per SM).
 // OZK: 0 for the lane build only; 16 or 32 for the instantiations with the
 // tensor-core build at that K (kept out of the other instantiations, whose
-// register allocation it would perturb, and with K fixed at compile time).
+// register allocation it would perturb, and with K fixed at compile time);
+// -1 for the FP64 contexts (no double-FP32 copy of g, the solves of
+// als_slow.cuh; never on a cluster).
 template <int MINB, bool SPLIT, int OZK>
 __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
+  constexpr bool F64 = OZK < 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   AlsShared& sm = *reinterpret_cast<AlsShared*>(smem_raw);
   const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
@@ -1164,7 +1172,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
   }
   // the tensor-core build (K = 16 or 32): its accumulator columns, held
   // until the last sweep (the address passes through red[0])
-  const bool oz = OZK != 0 && a.oz && a.K == OZK;
+  const bool oz = OZK > 0 && a.oz && a.K == OZK;
   uint32_t oz_tmem = 0;
   if (oz) {
     if (wid == 0) tc::tmem_alloc(reinterpret_cast<uint32_t*>(sm.red), OZ_TMEM_COLS);
@@ -1184,7 +1192,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
   __syncthreads();
   const float4 *gdf = nullptr, *gdfT = nullptr;
   int ge = 0;
-  if (a.df) {
+  if (!F64 && a.df) {
     gdf = a.gdf + item * (long long)ng * ng;
     gdfT = a.gdfT + item * (long long)ng * ng;
     ge = a.gscale[item];                                   // g is split by k_gsplit
@@ -1194,7 +1202,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
   const short* gexp = oz ? a.gexp + item * (long long)2 * K * ng : nullptr;
   // gx0 = g x0 (double-FP32 products on the mixed contexts), eps0 = x0^H g x0
   double e0 = 0.0;
-  if (a.df) {
+  if (!F64 && a.df) {
     als_gmat_df(sm, a, gdf, ge, x0, gx0 - rank * (long long)ng, ng, ng, item, rank, split, phase);
     for (int r = tid; r < ng; r += NTU_CTA) e0 += cmulc(x0[r], gx0[r]).x;
   } else {
@@ -1224,7 +1232,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
       // every CTA of a cluster is done with its copy of the last reduced
       // metric before any writes the next one, and all blocks are in before
       // anyone reads
-      if constexpr (OZK != 0) {
+      if constexpr (OZK > 0) {
         if (split > 1) als_exchange(a, item, phase);
         const bool built = oz && als_reduced_oz<OZK>(sm, a, a.gmap, item, ge, side,
                                                      split > 1 ? gX0 : gX,
@@ -1238,7 +1246,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
           tc_dead = true;
           break;
         }
-      } else if (a.df) {
+      } else if (!F64 && a.df) {
         if (split > 1) als_exchange(a, item, phase);
         als_reduced_df<SPLIT>(sm, a, gdf, gdfT, ge, side, split > 1 ? gX0 : gX,
                               reinterpret_cast<float4*>(split > 1 ? gC0 : gC), rank, split, nA2);
@@ -1247,13 +1255,18 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
         als_reduced(sm, a, g, side, Tm, gX, jv, gx0);
       }
       als_source(sm, a, side, jv, gx0);
-      if (!als_solve_chol(sm, a, side, gX, gC, jv, tau_max)) {
-        als_mirror(gX, nA);
-        als_solve(sm, a, side, gX, jv, pv, tauv, dv, ev, log);
+      if (!als_solve_chol<F64>(sm, a, side, gX, gC, jv, tau_max)) {
+        if constexpr (F64) {
+          if (nA <= LOW_SH_MAX) als_solve_spectrum<true>(sm, a, side, gX, jv, pv, tauv, dv, ev, Tm, log);
+          else als_solve_spectrum<false>(sm, a, side, gX, jv, pv, tauv, dv, ev, Tm, log);
+        } else {
+          als_mirror(gX, nA);
+          als_solve(sm, a, side, gX, jv, pv, tauv, dv, ev, log);
+        }
       }
     }
   }
-  if (OZK != 0 && a.oz && a.K == OZK) {
+  if (OZK > 0 && a.oz && a.K == OZK) {
     // every MMA has retired before the accumulator columns are released
     const OzSmem os = oz_smem(&sm.S, sm.red);
     __syncthreads();
@@ -1279,7 +1292,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
   }
   __syncthreads();
   double eps = 0.0;
-  if (a.df) {
+  if (!F64 && a.df) {
     als_gmat_df(sm, a, gdf, ge, xv, gx0 - rank * (long long)ng, ng, ng, item, rank, split,
                 phase);                                    // gx0 is free by now
     for (int r = tid; r < ng; r += NTU_CTA) eps += cmulc(xv[r], gx0[r]).x;
@@ -1320,7 +1333,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
 template <int OZK>
 cudaError_t als_launch_impl(const AlsArgs& a, int n, int split, bool three, size_t smem,
                             cudaStream_t stream) {
-  if (split > 1) {
+  if constexpr (OZK >= 0) if (split > 1) {
     void (*ck)(AlsArgs) = k_als<2, true, OZK>;
     cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(ck, cudaFuncAttributePreferredSharedMemoryCarveout,

@@ -1,6 +1,6 @@
 // Shared-memory layout and launch arguments of the ALS kernel k_als
 // (als_kernel.cuh), and the launchers of its instantiations, one per
-// translation unit: the lane build of the reduced metric only, and the
+// translation unit: FP64, the lane build of the reduced metric only, and the
 // tensor-core build at K = 16 and at K = 32.
 #pragma once
 #include <cuda_runtime.h>
@@ -70,6 +70,8 @@ struct AlsArgs {
 // launch error.
 cudaError_t als_launch_lanes(const AlsArgs& a, int n, int split, bool three, size_t smem,
                              cudaStream_t stream);
+cudaError_t als_launch_fp64(const AlsArgs& a, int n, int split, bool three, size_t smem,
+                            cudaStream_t stream);
 cudaError_t als_launch_tc16(const AlsArgs& a, int n, int split, bool three, size_t smem,
                             cudaStream_t stream);
 cudaError_t als_launch_tc32(const AlsArgs& a, int n, int split, bool three, size_t smem,

@@ -416,7 +416,8 @@ cudaError_t launch_als(ntu_ctx* c, int n, const double2* g, const double2* RA,
   }
   const bool three =
       split == 1 && (c->tune.als_ctas_per_sm ? c->tune.als_ctas_per_sm == 3 : n > 2 * sms);
-  cudaError_t e = !a.oz ? als_launch_lanes(a, n, split, three, smk, c->stream)
+  cudaError_t e = !a.df ? als_launch_fp64(a, n, split, three, smk, c->stream)
+                  : !a.oz ? als_launch_lanes(a, n, split, three, smk, c->stream)
                   : P.K == 16 ? als_launch_tc16(a, n, split, three, smk, c->stream)
                               : als_launch_tc32(a, n, split, three, smk, c->stream);
   if (e != cudaSuccess) return e;
