@@ -310,6 +310,7 @@ int ntu::init_context(const ntu_config* cfg, void* stream, ntu_ctx** out, int ma
       return fail(nullptr, st, "tensor maps of the split operands");
     }
   }
+  oz64_init(c);
   if (c->w.gsl) {
     // the tensor-core ALS build needs tcgen05 (compute capability 10.x)
     int major = 0, dev = 0;

@@ -437,6 +437,7 @@ int plan_build(ntu_ctx* c) {
 }
 
 void plan_free(ntu_ctx* c) {
+  oz64_free(c);
   if (c->plan.d_tab) cudaFree(c->plan.d_tab);
   c->plan.d_tab = nullptr;
 }
@@ -499,6 +500,39 @@ static cudaError_t env_chain(ntu_ctx* c, int n, const void* Ta, const void* Tb, 
   RG(run_gemm<C2>(c, P.t2, n, W.ETR, W.T1, W.T2));
   RG(run_gemm<C2>(c, P.h, n, W.EBR, W.T2, W.HR));
   RG(run_gemm<C2>(c, P.join, n, W.HL, W.HR, graw));
+  return cudaSuccess;
+}
+
+// The FP64 environment on the tensor cores: the products with long sums or
+// large results as sliced GEMMs (k_oz64.cu), in passes over as many items as the
+// slice scratch holds; the side edges and Y (sums of D terms) stay on the FP64
+// pipe.  The items of a pass use the first items of the intermediates.
+static cudaError_t env_chain_oz64(ntu_ctx* c, int n, const double2* Ta, const double2* Tb,
+                                  const double2* QA, const double2* QB, double2* graw) {
+  const Plan& P = c->plan;
+  Work& W = c->w;
+  double2 *EL = (double2*)W.EL, *ER = (double2*)W.ER, *Y = (double2*)W.Y, *T1 = (double2*)W.T1,
+          *T2 = (double2*)W.T2, *HL = (double2*)W.HL, *HR = (double2*)W.HR;
+  for (int i0 = 0; i0 < n; i0 += P.oz64.items) {
+    const int m = n - i0 < P.oz64.items ? n - i0 : P.oz64.items;
+    const double2 *ta = Ta + i0 * P.szT, *tb = Tb + i0 * P.szT;
+    const double2 *qa = QA + i0 * P.szQ, *qb = QB + i0 * P.szQ;
+    RG(run_gram<double2>(c, P.eL, m, tb, EL));
+    RG(run_gram<double2>(c, P.eR, m, ta, ER));
+    RG(launch_oz64(c, P.eTL, 0, m, tb, tb, (double2*)W.ETL));
+    RG(launch_oz64(c, P.eBL, 0, m, tb, tb, (double2*)W.EBL));
+    RG(launch_oz64(c, P.eTR, 0, m, ta, ta, (double2*)W.ETR));
+    RG(launch_oz64(c, P.eBR, 0, m, ta, ta, (double2*)W.EBR));
+    RG(run_gemm<double2>(c, P.y, m, qa, EL, Y));
+    RG(launch_oz64(c, P.t1, 1, m, Y, qa, T1));
+    RG(launch_oz64(c, P.t2, 2, m, (double2*)W.ETL, T1, T2));
+    RG(launch_oz64(c, P.h, 2, m, (double2*)W.EBL, T2, HL));
+    RG(run_gemm<double2>(c, P.y, m, qb, ER, Y));
+    RG(launch_oz64(c, P.t1, 1, m, Y, qb, T1));
+    RG(launch_oz64(c, P.t2, 2, m, (double2*)W.ETR, T1, T2));
+    RG(launch_oz64(c, P.h, 2, m, (double2*)W.EBR, T2, HR));
+    RG(launch_oz64(c, P.join, 3, m, HL, HR, graw + i0 * P.szG));
+  }
   return cudaSuccess;
 }
 
@@ -643,7 +677,9 @@ cudaError_t launch_env(ntu_ctx* c, int n, const double2* Ta, const double2* Tb,
                        const double2* QA, const double2* QB, void* graw) {
   const Plan& P = c->plan;
   Work& W = c->w;
-  if (c->cfg.precision == NTU_FP64) return env_chain<double2>(c, n, Ta, Tb, QA, QB, graw);
+  if (c->cfg.precision == NTU_FP64)
+    return P.oz64.items > 0 ? env_chain_oz64(c, n, Ta, Tb, QA, QB, (double2*)graw)
+                            : env_chain<double2>(c, n, Ta, Tb, QA, QB, graw);
   RG(to_f32(c, (long long)n * P.szT, Ta, W.Tac));
   RG(to_f32(c, (long long)n * P.szT, Tb, W.Tbc));
   RG(to_f32(c, (long long)n * P.szQ, QA, W.QAc));

@@ -52,6 +52,23 @@ struct TcOp {
   int mode, mtiles;
 };
 
+// FP64 GEMMs on the tensor cores by slicing (k_oz64.cu): operand geometry of
+// one plan GEMM (rowsA real rows of the doubled left operand, rowsB rows of the
+// right one, Kh padded complex terms) and the scratch shared by all of them.
+constexpr int OZ64_SLICES = 7;
+struct Oz64Geo {
+  int Kh, rowsA, rowsB;
+  CUtensorMap mapA, mapB;
+};
+struct Oz64 {
+  int items;                            // items per pass; 0: not available
+  Oz64Geo geo[4];                       // edges, t1, t2 and h, join
+  void* base;
+  char *SA, *SB;                        // slices of the left and the right operands
+  int *eA, *eB;                         // row exponents
+  unsigned* mx;                         // row maxima (long rows)
+};
+
 struct Plan {
   int D, d, d_anc, dp, r, K, m, ng, nA;
   long long szT, szQ, szR, szE1, szE2, szS2, szG;
@@ -68,6 +85,7 @@ struct Plan {
   long long rowsE, rowsT, rowsHL, rowsHR;  // allocated rows of the split operands
   int* d_tab;                           // device index tables
   int n_tab;
+  Oz64 oz64;                            // FP64 environment on the tensor cores
   // tensor-core build of the ALS reduced metric (K = 16, mixed contexts)
   int oz_ok;
   CUtensorMap mapGsl;                   // slices of g, box 128 rows x 64 BF16
@@ -156,6 +174,12 @@ int fail(ntu_ctx* c, int status, const char* fmt, ...);
 // Called after every launch: counts it and, in debug mode, synchronises and
 // reports the first failing kernel by name.
 cudaError_t after_launch(ntu_ctx* c, const char* name);
+
+// FP64 environment GEMMs on the tensor cores (k_oz64.cu)
+void oz64_init(ntu_ctx* c);
+void oz64_free(ntu_ctx* c);
+cudaError_t launch_oz64(ntu_ctx* c, const GemmOp& op, int gi, int n, const double2* A,
+                        const double2* B, double2* C);
 
 // plans and tables (k_env.cu)
 int plan_build(ntu_ctx* c);
