@@ -1017,41 +1017,10 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
   // BF16 in the next bond's environment: the arithmetic of these solves is
   // kept to the last bit.  A Cholesky factorisation of gX - sigma I proves the
   // same bound.
-  for (int idx = tid; idx < nA * nA; idx += NTU_CTA)
-    if (idx % nA >= idx / nA) gC[idx] = gX[idx];
+  const int ok = nA <= LOW_SH_MAX ? als_solve_fixpoint<true>(sm, nA, M0, gX, gC, jv, sigma)
+                                  : als_solve_fixpoint<false>(sm, nA, M0, gX, gC, jv, sigma);
   __syncthreads();
-  if (!cta_cholesky(gC, nA, sigma, &sm.flag)) return 0;
-  if (wid == 0) {
-    const double2* M0 = side == 0 ? sm.MA : sm.MB;
-    for (int i = lid; i < nA; i += 32) sm.y[i] = M0[i];     // warm start
-    __syncwarp();
-    int conv = 0;
-    double prev = INFINITY;
-    for (int it = 0; it < 60 && !conv; ++it) {
-      for (int i = lid; i < nA; i += 32) {
-        double2 v = sm.y[i], j = jv[i];
-        sm.y2[i] = make_double2(fma(-sigma, v.x, j.x), fma(-sigma, v.y, j.y));
-      }
-      __syncwarp();
-      warp_cholesky_solve(gC, nA, sm.y2);
-      double diff = 0.0, vmax = 0.0;
-      for (int i = lid; i < nA; i += 32) {
-        double2 n = sm.y2[i], o = sm.y[i];
-        diff = fmax(diff, fabs(n.x - o.x) + fabs(n.y - o.y));
-        vmax = fmax(vmax, fabs(n.x) + fabs(n.y));
-        sm.y[i] = n;
-      }
-      diff = warp_max(diff);
-      vmax = warp_max(vmax);
-      __syncwarp();
-      if (diff <= 1e-15 * vmax) conv = 1;                         // converged
-      else if (it >= 3 && diff >= 0.5 * prev && diff <= 1e-13 * vmax) conv = 1;  // rounding floor
-      prev = diff;
-    }
-    if (lid == 0) sm.flag = conv;
-  }
-  __syncthreads();
-  if (!sm.flag) return 0;
+  if (!ok) return 0;
   double2* M = side == 0 ? sm.MA : sm.MB;
   for (int i = tid; i < nA; i += NTU_CTA) M[i] = sm.y[i];
   if (tid == 0) { sm.tau_sel = tau_max; sm.n_fast += 1; }
