@@ -393,6 +393,7 @@ int plan_build(ntu_ctx* c) {
     const int hcolR = T.add({{K, 1}, {K, K}, {D, 0}, {D, 0}});
     h.mtiles = (int)(P.rowsE / 128);
     h.args.kTiles = (int)(P.krpE / 64); h.args.krp = (int)P.krpE;
+    h.args.kv = (int)D2; h.args.kim = (int)P.krpE / 2;
     h.args.Mc = (int)D2; h.args.N = (int)D2K2;
     h.args.pitch = pJ; h.args.krp_out = (int)P.krpJ;
     P.tc_hL = h;
@@ -406,6 +407,7 @@ int plan_build(ntu_ctx* c) {
     jn.mode = 0;
     jn.mtiles = (int)(P.rowsHL / 128);
     jn.args.kTiles = (int)(P.krpJ / 64); jn.args.krp = (int)P.krpJ;
+    jn.args.kv = (int)(2 * D4); jn.args.kim = 0;
     jn.args.Mc = (int)K2; jn.args.N = (int)K2;
     jn.args.sOut = P.szG;
     P.tc_join = jn;

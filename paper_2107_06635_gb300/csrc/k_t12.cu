@@ -94,8 +94,53 @@ struct T12Args {
   int* err;
 };
 
-// DT = 8: bond dimension fixed at compile time (every index of the epilogues
-// folds into constants); DT = 0: any D <= 8 at run time.
+// Epilogue 1 at a bond dimension fixed at compile time (D < 8): the columns
+// CS .. CS + 31 of accumulator 1 of one row (u, n), Re or Im, into the operand
+// buffer B2 (row n' D + n, K position k0 + u'), hi tile and lo tile 2 B_TILE on.
+// With D even a pair u', u' + 1 is one 4-byte store.
+template <int DT, int CS>
+__device__ __forceinline__ void epi1_cols(uint32_t taddr, bool rv, unsigned char* B2, int nn, int k0) {
+  constexpr int D2 = DT * DT;
+#pragma unroll
+  for (int c0 = CS; c0 < CS + 32; c0 += 16) {
+    if (c0 < D2) {
+      float v[16];
+      tc::tmem_ld16(taddr + (uint32_t)c0, v);
+      if (rv) {
+#pragma unroll
+        for (int q = 0; q < 16; q += 2) {
+          const int c = c0 + q;
+          if (c >= D2) break;
+          __nv_bfloat16 h0, l0, h1, l1;
+          split_bf16(v[q], h0, l0);
+          split_bf16(v[q + 1], h1, l1);
+          const int brow = c / DT * DT + nn, kre = k0 + c % DT;
+          unsigned char* t = B2 + (kre >> 6) * B_TILE;
+          const uint32_t off = swz(brow, kre & 63);
+          if (DT % 2 == 0) {
+            *reinterpret_cast<uint32_t*>(t + off) = pack_bf16(h0, h1);
+            *reinterpret_cast<uint32_t*>(t + 2 * B_TILE + off) = pack_bf16(l0, l1);
+          } else {
+            *reinterpret_cast<__nv_bfloat16*>(t + off) = h0;
+            *reinterpret_cast<__nv_bfloat16*>(t + 2 * B_TILE + off) = l0;
+            if (c + 1 < D2) {
+              const int brow1 = (c + 1) / DT * DT + nn, kre1 = k0 + (c + 1) % DT;
+              unsigned char* t1 = B2 + (kre1 >> 6) * B_TILE + swz(brow1, kre1 & 63);
+              *reinterpret_cast<__nv_bfloat16*>(t1) = h1;
+              *reinterpret_cast<__nv_bfloat16*>(t1 + 2 * B_TILE) = l1;
+            }
+          }
+        }
+      }
+    }
+  }
+}
+
+// DT > 0: bond dimension fixed at compile time (every index of the epilogues
+// folds into constants), DT = 8 also with paired units; DT = 0: any D <= 8 at
+// run time (D = 1, 2, and unpaired D = 8).  Run-time indices cost the epilogues
+// a division and a 2-byte store per value: 304 items at D = 6 took 1.37 ms a
+// launch with them.
 template <int DT>
 __global__ void __launch_bounds__(T12_THREADS, 1) k_t12(const __grid_constant__ CUtensorMap mA1,
                                                       const __grid_constant__ CUtensorMap mB1,
@@ -244,6 +289,10 @@ __global__ void __launch_bounds__(T12_THREADS, 1) k_t12(const __grid_constant__ 
             const uint64_t bl = tc::sdesc_k128(tc::smem_u32(B2 + (2 + c) * tstride));
 #pragma unroll
             for (int kk4 = 0; kk4 < 4; ++kk4) {
+              // the factors occupy K positions 0 .. and krpE/2 .. (D^2 each);
+              // steps of zeros only are left out (adding zero changes no bit)
+              const int pos = c * 64 + kk4 * 16, im0 = a.krpE / 2;
+              if (DT != 8 && pos >= D2 && (pos + 16 <= im0 || pos >= im0 + D2)) continue;
               tc::mma_bf16_ts(acc, ah + 8 * kk4, bh + 2 * kk4, id2, (c | kk4) != 0);
               tc::mma_bf16_ts(acc, ah + 8 * kk4, bl + 2 * kk4, id2, 1);
               tc::mma_bf16_ts(acc, al + 8 * kk4, bh + 2 * kk4, id2, 1);
@@ -327,6 +376,11 @@ __global__ void __launch_bounds__(T12_THREADS, 1) k_t12(const __grid_constant__ 
             *reinterpret_cast<uint4*>(dst + 2 * TS) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
           }
         }
+      } else if constexpr (DT > 0) {
+        const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 64);
+        const int k0 = im * half + uu * D;
+        if (cs == 0) epi1_cols<DT, 0>(ta, rv, B2, nn, k0);
+        else epi1_cols<DT, 32>(ta, rv, B2, nn, k0);
       } else
 #pragma unroll 1
       for (int c0 = cs; c0 < cs + 32; c0 += 16) {
@@ -470,11 +524,25 @@ __global__ void __launch_bounds__(T12_THREADS, 1) k_t12(const __grid_constant__ 
 
 size_t t12_smem_bytes() { return T12_SMEM; }
 
+typedef void (*T12Kernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, T12Args);
+static T12Kernel t12_kernel(int D, bool pair) {
+  switch (D) {
+    case 3: return k_t12<3>;
+    case 4: return k_t12<4>;
+    case 5: return k_t12<5>;
+    case 6: return k_t12<6>;
+    case 7: return k_t12<7>;
+    default: return D == 8 && pair ? k_t12<8> : k_t12<0>;
+  }
+}
+
 cudaError_t t12_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(k_t12<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)T12_SMEM);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_t12<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T12_SMEM);
+  for (int D = 2; D <= 8; ++D) {
+    cudaError_t e = cudaFuncSetAttribute(t12_kernel(D, true), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)T12_SMEM);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Etop: the split top edge of this half (W.ETLd or W.ETRd, doubled A
@@ -494,10 +562,8 @@ cudaError_t launch_t12(ntu_ctx* c, int n, const void* Etop) {
   a.err = c->d_status;
   if (a.units == 0) return cudaSuccess;
   const int grid = (int)(a.units < c->sms ? a.units : c->sms);
-  if (P.D == 8 && c->tune.t12_pair != 0)
-    k_t12<8><<<grid, T12_THREADS, T12_SMEM, c->stream>>>(P.mapYs, P.mapQs, P.mapT2st, a);
-  else
-    k_t12<0><<<grid, T12_THREADS, T12_SMEM, c->stream>>>(P.mapYs, P.mapQs, P.mapT2st, a);
+  t12_kernel(P.D, c->tune.t12_pair != 0)<<<grid, T12_THREADS, T12_SMEM, c->stream>>>(
+      P.mapYs, P.mapQs, P.mapT2st, a);
   return after_launch(c, "k_t12");
 }
 

@@ -154,6 +154,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_gemm(const __grid_constant
           const uint64_t bl = tc::sdesc_k128(tc::smem_u32(sB + sl * TILE_B));
 #pragma unroll
           for (int kk = 0; kk < TBK / 16; ++kk) {
+            // steps of padding only are left out (adding zero changes no bit)
+            const int pos = (it >> 1) * TBK + 16 * kk;
+            if (pos >= a.kv && (pos + 16 <= a.kim || pos >= a.kim + a.kv)) continue;
             tc::mma_bf16(acc, ah + 2 * kk, bh + 2 * kk, idesc, (it | kk) != 0);
             tc::mma_bf16(acc, ah + 2 * kk, bl + 2 * kk, idesc, 1);
             tc::mma_bf16(acc, al + 2 * kk, bh + 2 * kk, idesc, 1);

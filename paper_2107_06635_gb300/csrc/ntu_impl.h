@@ -32,6 +32,7 @@ struct GemmOp {
 struct TcArgs {
   int kTiles;            // 64-wide K tiles per split pass
   int krp;               // padded real K of one half ([hi | lo] rows are 2 krp wide)
+  int kv, kim;           // K positions 0 .. kv - 1 and kim .. kim + kv - 1 hold data
   int Mc, N;             // valid complex rows, valid columns
   int mtiles;            // 128-row tiles of the doubled A operand
   const int *rowC, *colC, *rowK, *colK;
