@@ -25,11 +25,225 @@ __device__ __forceinline__ double2 ld2(const float2* p) {
 // g <- (g + g^H)/2.  g is positive definite, and clipping its negative
 // eigenvalues would change nothing, when the Gershgorin discs of the rows
 // lie right of zero (min_i d_i - s_i > 0, s_i = sum_{j != i} |Re| + |Im| >=
-// sum_{j != i} |g_ij|) or, failing that, when a Cholesky factorisation of g
+// sum_{j != i} |g_ij|) or, failing that, when a triangular factorisation of g
 // succeeds; otherwise g = W diag(max(lambda, 0)) W^H from a full
 // eigendecomposition.  Finally g /= trace(g).
 // diag = [||g - g^H|| / ||g||, lambda_min / lambda_max (NaN on the two
 // certified paths), log(trace)].
+//
+// The discs decide almost every metric of a batch, so they are taken grid-wide
+// in three streaming kernels: row statistics (a block per 32 rows; the entries
+// (c, r) come in 32 x 32 tiles turned in shared memory), the decision (a block
+// per item) and the scaled result (a block per pair of mirrored tiles).  One
+// block per item with strided reads of the mirrored entries held a K = 32
+// metric for 4 ms on one SM; now 45 of them take 0.65 ms, 912 at K = 16 0.90
+// against 1.24 ms.  k_repair then runs for the undecided items only.
+struct RowStat {
+  double d, lo;                 // diagonal entry, disc's left end
+};
+
+template <typename C2in>
+__global__ void __launch_bounds__(256) k_herm_stats(int ng, const C2in* __restrict__ graw,
+                                                    RowStat* __restrict__ rows,
+                                                    double2* __restrict__ part) {
+  constexpr bool F32 = std::is_same<C2in, float2>::value;
+  typedef typename std::conditional<F32, float, double>::type R;
+  __shared__ C2in tb[32][33];
+  __shared__ double red[2 * NTU_WARPS];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r0 = blockIdx.x * 32;
+  const long long item = blockIdx.y;
+  const C2in* gr = graw + item * (long long)ng * ng;
+  C2in zero;
+  zero.x = 0; zero.y = 0;
+  R sr[4] = {0, 0, 0, 0}, n2 = 0, h2 = 0;
+  double dr[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int c0 = 0; c0 < ng; c0 += 32) {
+    C2in a[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = r0 + w + 8 * i, c = c0 + w + 8 * i;
+      a[i] = r < ng && c0 + lane < ng ? gr[(size_t)r * ng + c0 + lane] : zero;
+      tb[w + 8 * i][lane] = c < ng && r0 + lane < ng ? gr[(size_t)c * ng + r0 + lane] : zero;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const C2in b = tb[lane][w + 8 * i];                   // entry (c, r)
+      const R dx = a[i].x - b.x, dy = a[i].y + b.y;
+      n2 = fma(a[i].x, a[i].x, fma(a[i].y, a[i].y, n2));
+      h2 = fma(dx, dx, fma(dy, dy, h2));
+      if (r0 + w + 8 * i == c0 + lane) dr[i] = (double)a[i].x;
+      else sr[i] += (R)0.5 * (fabs(a[i].x + b.x) + fabs(a[i].y - b.y));
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = r0 + w + 8 * i;
+    const double d = warp_sum(dr[i]);                       // one lane holds it
+    // relative rounding of the radius below 2e-5 in FP32 (n_g <= 1024 terms)
+    const double s = F32 ? (double)warp_sum_f((float)sr[i]) * (1.0 + 1e-4)
+                         : warp_sum((double)sr[i]) * (1.0 + 1e-12);
+    if (lane == 0 && r < ng) rows[item * ng + r] = RowStat{d, d - s};
+  }
+  const double2 t = block_sum2(make_double2((double)n2, (double)h2), red);
+  if (threadIdx.x == 0) part[item * ng + blockIdx.x] = t;
+}
+
+// scale[item] = 1 / (2 tr) where the discs decide, else 0.  The trace is
+// summed as k_repair sums it (rows r, r + 8, ... by warp, then the warps).
+__global__ void __launch_bounds__(NTU_CTA) k_herm_decide(int ng, const RowStat* __restrict__ rows,
+                                                         const double2* __restrict__ part,
+                                                         double* __restrict__ scale,
+                                                         double* __restrict__ trace,
+                                                         double* __restrict__ diag, int* paths) {
+  __shared__ double red[2 * NTU_WARPS], tw[NTU_WARPS];
+  const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
+  const long long item = blockIdx.x;
+  const RowStat* rs = rows + item * ng;
+  double lo = INFINITY;
+  for (int r = tid; r < ng; r += NTU_CTA) lo = fmin(lo, rs[r].lo);
+  lo = block_min(lo, red);
+  if (lid == 0) {
+    double t = 0.0;
+    for (int r = wid; r < ng; r += NTU_WARPS) t += rs[r].d;
+    tw[wid] = t;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double tr = 0.0, n2 = 0.0, h2 = 0.0;
+    for (int w = 0; w < NTU_WARPS; ++w) tr += tw[w];
+    for (int b = 0; b < (ng + 31) / 32; ++b) { n2 += part[item * ng + b].x; h2 += part[item * ng + b].y; }
+    const bool ok = lo > 0.0 && isfinite(lo) && tr > 0.0 && isfinite(tr);
+    scale[item] = ok ? 0.5 / tr : 0.0;
+    trace[item] = tr;
+    diag[item * 3 + 0] = n2 > 0.0 ? sqrt(h2 / n2) : 0.0;
+    if (ok) {
+      if (paths) atomicAdd(paths + 3, 1);
+      diag[item * 3 + 1] = __longlong_as_double(0x7ff8000000000000ULL);   // NaN
+      diag[item * 3 + 2] = log(tr);
+    }
+  }
+}
+
+// The decided items: g = (graw + graw^H) / (2 tr), tile (I, J), I >= J, and its
+// mirror image, turned in shared memory: each pair of entries is converted and
+// scaled once (FP64 operations and conversions bound this kernel).
+template <typename C2in>
+__global__ void __launch_bounds__(256) k_herm_write(int ng, const C2in* __restrict__ graw,
+                                                    const double* __restrict__ scale,
+                                                    double2* __restrict__ g) {
+  __shared__ double2 t[32][33];
+  const long long item = blockIdx.y;
+  const double hinv = scale[item];
+  if (hinv == 0.0) return;
+  int I = (int)((sqrtf(8.0f * (float)blockIdx.x + 1.0f) - 1.0f) * 0.5f);
+  while ((I + 1) * (I + 2) / 2 <= (int)blockIdx.x) ++I;
+  while (I > 0 && I * (I + 1) / 2 > (int)blockIdx.x) --I;
+  const int J = (int)blockIdx.x - I * (I + 1) / 2;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, r0 = I * 32, c0 = J * 32;
+  const C2in* gr = graw + item * (long long)ng * ng;
+  double2* gi = g + item * (long long)ng * ng;
+  C2in* tb = reinterpret_cast<C2in*>(&t[0][0]);             // [32][33] of the raw type first
+  C2in a[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int k = w + 8 * i;
+    if (r0 + k < ng && c0 + lane < ng) a[i] = gr[(size_t)(r0 + k) * ng + c0 + lane];
+    if (c0 + k < ng && r0 + lane < ng) tb[k * 33 + lane] = gr[(size_t)(c0 + k) * ng + r0 + lane];
+  }
+  __syncthreads();
+  double2 h[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int k = w + 8 * i;
+    if (r0 + k < ng && c0 + lane < ng) {
+      const double2 u = ld2(&a[i]), v = ld2(&tb[lane * 33 + k]);
+      h[i] = make_double2((u.x + v.x) * hinv, (u.y - v.y) * hinv);
+      gi[(size_t)(r0 + k) * ng + c0 + lane] = h[i];
+    }
+  }
+  if (I == J) return;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) t[w + 8 * i][lane] = h[i];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int k = w + 8 * i;
+    if (c0 + k < ng && r0 + lane < ng) gi[(size_t)(c0 + k) * ng + r0 + lane] = cconj(t[lane][k]);
+  }
+}
+
+// Whether H - delta I (H row-major, Hermitian) has an L D L^H
+// factorisation in FP32, delta = 6 (n + 3) 2^-24 tr H: the rounding of the
+// factorisation is a perturbation of at most 4 (n + 2) 2^-24 |L| |D| |L|^H,
+// whose norm is below 4 (n + 2) 2^-24 tr H for a positive definite matrix, and
+// that of the entries below 2^-24 tr H, so success proves H positive definite.
+// It decides metrics with lambda_min above some 1e-4 tr H at 64 times the FP64
+// rate (n = 400: 3.1 ms, bound by the trailing columns' traffic to L2, where the
+// FP64 Cholesky held the SM's FP64 pipe for 21 ms); a warp per column, four rows
+// a lane in flight.
+// cert[item] = 1 where it succeeds; a block of CERT_THREADS per undecided item.
+constexpr int CERT_THREADS = 1024;
+template <typename C2in>
+__global__ void __launch_bounds__(CERT_THREADS) k_herm_certify(int n, const C2in* __restrict__ graw,
+                                                               const double* __restrict__ scale,
+                                                               const double* __restrict__ traces,
+                                                               double2* __restrict__ scr,
+                                                               int* __restrict__ cert) {
+  __shared__ float2 col[1024];                              // n_g <= 1024
+  const long long item = blockIdx.x;
+  const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
+  if (tid == 0) cert[item] = 0;
+  if (scale[item] != 0.0) return;                           // decided by the discs
+  const double trace = traces[item];
+  if (!(trace > 0x1p-900) || !(trace < 0x1p900)) return;
+  const double f = scalbn(1.0, -ilogb(trace)), delta = 6.0 * (n + 3) * 0x1p-24 * trace;
+  const C2in* gr = graw + item * (long long)n * n;
+  float2* A = reinterpret_cast<float2*>(scr + item * (long long)n * n);
+  for (int idx = tid; idx < n * n; idx += CERT_THREADS) {
+    const int k = idx / n, i = idx % n;                     // column k, row i: conj of (k, i)
+    if (i < k) continue;
+    const double2 a = ld2(gr + idx), b = ld2(gr + (size_t)i * n + k);
+    double hx = 0.5 * (a.x + b.x);
+    if (i == k) hx -= delta;
+    A[idx] = make_float2((float)(hx * f), (float)(-0.5 * (a.y - b.y) * f));
+  }
+  __syncthreads();
+  for (int j = 0; j < n; ++j) {
+    const float2* c = A + (size_t)j * n;
+    const float d = c[j].x;
+    if (!(d > 0.f) || !isfinite(d)) return;                 // the same in every thread
+    const float r = 1.0f / d;
+    for (int i = j + 1 + tid; i < n; i += CERT_THREADS) col[i] = c[i];
+    __syncthreads();
+    for (int k = j + 1 + wid; k < n; k += CERT_THREADS / 32) {   // a_ik -= c_i conj(c_k) / d
+      const float2 ck = col[k];
+      const float lx = ck.x * r, ly = ck.y * r;
+      float2* ak = A + (size_t)k * n;
+      for (int i0 = k + lid; i0 < n; i0 += 128) {
+        float2 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i0 + 32 * u < n) x[u] = ak[i0 + 32 * u];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + 32 * u;
+          if (i < n) {
+            const float2 ci = col[i];
+            x[u].x = fmaf(-ci.x, lx, fmaf(-ci.y, ly, x[u].x));
+            x[u].y = fmaf(-ci.y, lx, fmaf(ci.x, ly, x[u].y));
+            ak[i] = x[u];
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (tid == 0) cert[item] = 1;
+}
+
 template <typename C2in>
 __global__ void __launch_bounds__(NTU_CTA) k_repair(int ng, const C2in* __restrict__ graw,
                                                     double2* __restrict__ g,
@@ -40,103 +254,47 @@ __global__ void __launch_bounds__(NTU_CTA) k_repair(int ng, const C2in* __restri
                                                     double2* __restrict__ tau,
                                                     double2* __restrict__ pv,
                                                     double* __restrict__ diag, int* status,
-                                                    int* paths) {
+                                                    int* paths,
+                                                    const double* __restrict__ scale,
+                                                    const int* __restrict__ cert) {
+  if (scale[blockIdx.x] != 0.0) return;             // decided by the discs
   extern __shared__ __align__(16) double chain[];   // 2 * ng (also n_g float4 for the Cholesky)
   __shared__ double sred[2 * NTU_WARPS];
   __shared__ int sh[4];
   __shared__ int okflag;
-  const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
+  const int tid = threadIdx.x;
   const long long item = blockIdx.x;
   const size_t nn = (size_t)ng * ng;
   const C2in* gr = graw + item * nn;
   double2* gi = g + item * nn;
   double2* sc = scr + item * nn;
-  // 1. Hermiticity defect, Gershgorin discs and trace of the Hermitian part,
-  // one warp per row
-  double n2 = 0.0, h2 = 0.0, glo = INFINITY, trw = 0.0;
-  if (std::is_same<C2in, float2>::value) {
-    // FP32 raw metric (mixed contexts): the statistics and the disc radii in
-    // FP32 (relative rounding < 2e-5 for n_g <= 1024 terms, covered by
-    // inflating the radii by 1e-4); the diagonal Re g_rr is exact
-    const float2* gf = reinterpret_cast<const float2*>(gr);
-    for (int r = wid; r < ng; r += NTU_WARPS) {
-      float srf = 0.f, n2f = 0.f, h2f = 0.f;
-      double dr = 0.0;
-      for (int c = lid; c < ng; c += 32) {
-        const float2 a = gf[(size_t)r * ng + c], b = gf[(size_t)c * ng + r];
-        n2f = fmaf(a.x, a.x, fmaf(a.y, a.y, n2f));
-        const float dx = a.x - b.x, dy = a.y + b.y;
-        h2f = fmaf(dx, dx, fmaf(dy, dy, h2f));
-        if (c == r) dr = (double)a.x;
-        else srf += 0.5f * (fabsf(a.x + b.x) + fabsf(a.y - b.y));
-      }
-      n2 += (double)n2f;
-      h2 += (double)h2f;
-      srf = warp_sum_f(srf);
-      dr = warp_sum(dr);                 // one lane holds the diagonal
-      glo = fmin(glo, dr - (double)srf * (1.0 + 1e-4));
-      trw += dr;
-    }
-  } else {
-    for (int r = wid; r < ng; r += NTU_WARPS) {
-      double sr = 0.0, dr = 0.0;
-      for (int c = lid; c < ng; c += 32) {
-        double2 a = ld2(gr + (size_t)r * ng + c), b = ld2(gr + (size_t)c * ng + r);
-        double2 h = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
-        n2 += cabs2(a);
-        h2 += cabs2(make_double2(a.x - b.x, a.y + b.y));
-        if (c == r) dr = h.x;
-        else sr += fabs(h.x) + fabs(h.y);
-      }
-      sr = warp_sum(sr);
-      dr = warp_sum(dr);                 // one lane holds the diagonal
-      glo = fmin(glo, dr - sr * (1.0 + 1e-12));   // margin for the rounding of s
-      trw += dr;
-    }
-  }
-  if (lid != 0) trw = 0.0;
-  n2 = block_sum(n2, sred);
-  h2 = block_sum(h2, sred);
-  glo = block_min(glo, sred);
-  const double trg = block_sum(trw, sred);
-  const double herm = n2 > 0.0 ? sqrt(h2 / n2) : 0.0;
-  if (glo > 0.0 && isfinite(glo) && trg > 0.0 && isfinite(trg)) {
-    // certified by the discs: write (g + g^H) / (2 tr) directly
-    // (a + conj b) / 2 is exact in FP64; scaling by inv / 2 rounds once
-    const double hinv = 0.5 / trg;
-    for (size_t idx = tid; idx < nn; idx += NTU_CTA) {
-      int r = idx / ng, c = idx % ng;
-      double2 a = ld2(gr + idx), b = ld2(gr + (size_t)c * ng + r);
-      gi[idx] = make_double2((a.x + b.x) * hinv, (a.y - b.y) * hinv);
-    }
-    if (tid == 0) {
-      if (paths) atomicAdd(paths + 3, 1);
-      diag[item * 3 + 0] = herm;
-      diag[item * 3 + 1] = __longlong_as_double(0x7ff8000000000000ULL);   // NaN
-      diag[item * 3 + 2] = log(trg);
-    }
-    return;
-  }
-  // an FP32 raw metric (mixed contexts) is certified in double-FP32
-  // arithmetic, which resolves it far below its own rounding; FP64 otherwise
-  constexpr bool kDf = std::is_same<C2in, float2>::value;
   for (size_t idx = tid; idx < nn; idx += NTU_CTA) {
     int r = idx / ng, c = idx % ng;
     double2 a = ld2(gr + idx), b = ld2(gr + (size_t)c * ng + r);
-    double2 h = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
-    gi[idx] = h;
-    if (kDf) reinterpret_cast<float4*>(sc)[(size_t)c * ng + r] = df_split(h);
-    else sc[(size_t)c * ng + r] = h;     // column-major copy
+    gi[idx] = make_double2(0.5 * (a.x + b.x), 0.5 * (a.y - b.y));
   }
-  // 2. Cholesky of the lower triangle certifies positive definiteness
   __syncthreads();
-  int ok = kDf ? cta_cholesky_df(reinterpret_cast<float4*>(sc), ng, &okflag,
-                                 reinterpret_cast<float4*>(chain))
-               : cta_cholesky(sc, ng, 0.0, &okflag);
+  // 1. a triangular factorisation certifies positive definiteness: in FP32
+  // with room for its rounding (k_herm_certify), else in double-FP32 for an FP32 raw metric
+  // (mixed contexts; it resolves it far below its own rounding), in FP64
+  // otherwise
+  constexpr bool kDf = std::is_same<C2in, float2>::value;
+  int ok = cert[item];
+  if (!ok) {
+    for (size_t idx = tid; idx < nn; idx += NTU_CTA) {      // column-major copy
+      const size_t t = (idx % ng) * ng + idx / ng;
+      if (kDf) reinterpret_cast<float4*>(sc)[t] = df_split(gi[idx]);
+      else sc[t] = gi[idx];
+    }
+    __syncthreads();
+    ok = kDf ? cta_cholesky_df(reinterpret_cast<float4*>(sc), ng, &okflag,
+                               reinterpret_cast<float4*>(chain))
+             : cta_cholesky(sc, ng, 0.0, &okflag);
+  }
   if (tid == 0 && paths) atomicAdd(paths + (ok ? 4 : 5), 1);
   double ratio = __longlong_as_double(0x7ff8000000000000ULL);   // NaN
   if (!ok) {
-    // 3. full eigendecomposition and clipping of negative eigenvalues
+    // 2. full eigendecomposition and clipping of negative eigenvalues
     double2* ta = tau + item * ng;
     double2* pp = pv + item * ng;
     double* dd = de + item * 2 * ng;
@@ -183,7 +341,7 @@ __global__ void __launch_bounds__(NTU_CTA) k_repair(int ng, const C2in* __restri
     }
     __syncthreads();
   }
-  // 4. unit trace
+  // 3. unit trace
   double tr = 0.0;
   for (int i = tid; i < ng; i += NTU_CTA) tr += gi[(size_t)i * ng + i].x;
   tr = block_sum(tr, sred);
@@ -194,7 +352,6 @@ __global__ void __launch_bounds__(NTU_CTA) k_repair(int ng, const C2in* __restri
   const double inv = 1.0 / tr;
   for (size_t idx = tid; idx < nn; idx += NTU_CTA) gi[idx] = cscale(gi[idx], inv);
   if (tid == 0) {
-    diag[item * 3 + 0] = herm;
     diag[item * 3 + 1] = ratio;
     diag[item * 3 + 2] = log(tr);
   }
@@ -317,23 +474,39 @@ size_t als_smem_bytes() { return sizeof(AlsShared); }
 
 long long oz_rows_side(int K) { return oz_supported(K) ? oz_geo(K).rows_side : 0; }
 
-cudaError_t launch_repair(ntu_ctx* c, int n, const void* graw, int raw_is_f32, double2* g,
-                          double* diag) {
+template <typename C2in>
+static cudaError_t run_repair(ntu_ctx* c, int n, const C2in* graw, double2* g, double* diag) {
   const Plan& P = c->plan;
   Work& W = c->w;
-  size_t sm = 2 * sizeof(double) * P.ng;
-  if (raw_is_f32) {
-    cudaFuncSetAttribute(k_repair<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_repair<float2><<<n, NTU_CTA, sm, c->stream>>>(P.ng, (const float2*)graw, g, W.gscr, W.gw,
-                                                    W.gz, W.geig, W.gtau, W.gp, diag, c->d_status,
-                                                    c->d_paths);
-  } else {
-    cudaFuncSetAttribute(k_repair<double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_repair<double2><<<n, NTU_CTA, sm, c->stream>>>(P.ng, (const double2*)graw, g, W.gscr,
-                                                     W.gw, W.gz, W.geig, W.gtau, W.gp, diag,
-                                                     c->d_status, c->d_paths);
-  }
+  RowStat* rows = reinterpret_cast<RowStat*>(W.gtau);       // n_g entries of 16 bytes per item
+  double* scale = reinterpret_cast<double*>(W.x0);          // ALS scratch, free here
+  double* trace = scale + n;
+  const int nb = (P.ng + 31) / 32;
+  k_herm_stats<C2in><<<dim3((unsigned)nb, (unsigned)n), 256, 0, c->stream>>>(P.ng, graw, rows, W.gp);
+  cudaError_t e = after_launch(c, "k_herm_stats");
+  if (e != cudaSuccess) return e;
+  k_herm_decide<<<n, NTU_CTA, 0, c->stream>>>(P.ng, rows, W.gp, scale, trace, diag, c->d_paths);
+  e = after_launch(c, "k_herm_decide");
+  if (e != cudaSuccess) return e;
+  k_herm_write<C2in><<<dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)n), 256, 0, c->stream>>>(
+      P.ng, graw, scale, g);
+  e = after_launch(c, "k_herm_write");
+  if (e != cudaSuccess) return e;
+  int* cert = reinterpret_cast<int*>(W.gx0);                // ALS scratch, free here
+  k_herm_certify<C2in><<<n, CERT_THREADS, 0, c->stream>>>(P.ng, graw, scale, trace, W.gscr, cert);
+  e = after_launch(c, "k_herm_certify");
+  if (e != cudaSuccess) return e;
+  const size_t sm = 2 * sizeof(double) * P.ng;
+  cudaFuncSetAttribute(k_repair<C2in>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  k_repair<C2in><<<n, NTU_CTA, sm, c->stream>>>(P.ng, graw, g, W.gscr, W.gw, W.gz, W.geig, W.gtau,
+                                                W.gp, diag, c->d_status, c->d_paths, scale, cert);
   return after_launch(c, "k_repair");
+}
+
+cudaError_t launch_repair(ntu_ctx* c, int n, const void* graw, int raw_is_f32, double2* g,
+                          double* diag) {
+  return raw_is_f32 ? run_repair(c, n, (const float2*)graw, g, diag)
+                    : run_repair(c, n, (const double2*)graw, g, diag);
 }
 
 cudaError_t launch_als(ntu_ctx* c, int n, const double2* g, const double2* RA,
