@@ -136,6 +136,130 @@ k_cgemm(GemmArgs g, const C2* __restrict__ A, const C2* __restrict__ B, C2* __re
   }
 }
 
+// FP32 products of the NTU_MIXED_FP32 environment.  The sums run over k in
+// order with the operations of k_cgemm, so the results are the same bits for
+// every tile.  Bound by the FP32 pipe (4 FMAs a complex term).  A warp holds TM
+// rows of 32 TN columns (rows broadcast, columns conflict-free from shared
+// memory: TM + TN 8-byte loads per 4 TM TN FMAs), 16 terms a stage, up to three
+// stages in flight by cp.async, only as many terms as there are: k_cgemm loads
+// between two barriers with nothing in flight, pads 14 or 49 terms to 16 or 64
+// and 49 or 196 rows to 64 or 256.  The tile is the one with the fewest
+// padded multiply-adds (cgemm32_pick).
+__device__ __forceinline__ void cp_async8(void* dst, const void* src, bool on) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(on ? 8 : 0)
+               : "memory");
+}
+
+constexpr int C32_BK = 16, C32_STAGES = 3;
+
+template <int TM, int TN, bool CB>
+__global__ void __launch_bounds__(256, 2)
+k_cgemm32(GemmArgs g, const float2* __restrict__ A, const float2* __restrict__ B,
+          float2* __restrict__ C) {
+  constexpr int BM = 8 * TM, BN = 32 * TN, BK = C32_BK, STG = BK * (BM + BN);
+  extern __shared__ __align__(16) float2 c32_smem[];
+  __shared__ int rA[BM], cB[BN];
+  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+  const long long b = blockIdx.z;
+  const float2* Ab = A + b * g.sA;
+  const float2* Bb = B + b * g.sB;
+  float2* Cb = C + b * g.sC;
+  for (int i = tid; i < BM; i += 256) rA[i] = (m0 + i < g.M) ? g.rowA[m0 + i] : -1;
+  for (int i = tid; i < BN; i += 256) cB[i] = (n0 + i < g.N) ? g.colB[n0 + i] : -1;
+  float2 acc[TM][TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  __syncthreads();
+  const int chunks = (g.Kd + BK - 1) / BK;
+  auto load = [&](int ch) {
+    if (ch < chunks) {
+      float2* as = c32_smem + (ch % C32_STAGES) * STG;
+      float2* bs = as + BK * BM;
+      const int k0 = ch * BK, kc = min(BK, g.Kd - k0);
+#pragma unroll 2
+      for (int i = tid; i < kc * BM; i += 256) {
+        const int r = rA[i % BM];
+        cp_async8(as + i, Ab + (r >= 0 ? (long long)r + g.kA[k0 + i / BM] : 0), r >= 0);
+      }
+#pragma unroll 2
+      for (int i = tid; i < kc * BN; i += 256) {
+        const int r = cB[i % BN];
+        cp_async8(bs + i, Bb + (r >= 0 ? (long long)r + g.kB[k0 + i / BN] : 0), r >= 0);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int s = 0; s < C32_STAGES - 1; ++s) load(s);
+  for (int ch = 0; ch < chunks; ++ch) {
+    load(ch + C32_STAGES - 1);                          // its stage was read before the last barrier
+    asm volatile("cp.async.wait_group %0;" ::"n"(C32_STAGES - 1) : "memory");
+    __syncthreads();
+    const float2* as = c32_smem + (ch % C32_STAGES) * STG + ty * TM;
+    const float2* bs = c32_smem + (ch % C32_STAGES) * STG + BK * BM + tx;
+    const int kc = min(BK, g.Kd - ch * BK);
+#pragma unroll 2
+    for (int kk = 0; kk < kc; ++kk) {
+      float2 x[TM], y[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) x[i] = as[kk * BM + i];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        y[j] = bs[kk * BN + 32 * j];
+        if (CB) y[j].y = -y[j].y;
+      }
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) {
+          float re = acc[i][j].x, im = acc[i][j].y;
+          re = fmaf(x[i].x, y[j].x, re); re = fmaf(-x[i].y, y[j].y, re);
+          im = fmaf(x[i].x, y[j].y, im); im = fmaf(x[i].y, y[j].x, im);
+          acc[i][j] = make_float2(re, im);
+        }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < TM; ++i) {
+    const int m = m0 + ty * TM + i;
+    if (m >= g.M) break;
+    const long long rc = g.rowC[m];
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int n = n0 + tx + 32 * j;
+      if (n < g.N) Cb[rc + g.colC[n]] = acc[i][j];
+    }
+  }
+}
+
+typedef void (*Cgemm32)(GemmArgs, const float2*, const float2*, float2*);
+struct Cgemm32Tile { int tm, tn; Cgemm32 fn[2]; };          // fn[conjB]
+#define C32(TM, TN) {TM, TN, {k_cgemm32<TM, TN, false>, k_cgemm32<TM, TN, true>}}
+static const Cgemm32Tile c32_tiles[] = {C32(2, 2), C32(4, 2), C32(5, 2), C32(7, 2), C32(8, 2), C32(4, 4),
+                                        C32(5, 4), C32(7, 4), C32(8, 4), C32(5, 7), C32(6, 5)};
+#undef C32
+
+// The tile with the least time by count: waves of two CTAs per SM times the
+// multiply-adds of a tile (rows and columns padded to it), times 1 + (shared
+// loads per FMA).  Few products thus go to small tiles on many SMs.
+static const Cgemm32Tile& cgemm32_pick(int M, int N, long long items, int sms) {
+  const Cgemm32Tile* best = c32_tiles;
+  double cost = 0.0;
+  for (const Cgemm32Tile& t : c32_tiles) {
+    const long long bm = 8 * t.tm, bn = 32 * t.tn;
+    const long long ctas = (M + bm - 1) / bm * ((N + bn - 1) / bn) * items;
+    const double c = (double)((ctas + 2 * sms - 1) / (2 * sms)) * (double)(bm * bn) *
+                     (1.0 + (double)(t.tm + t.tn) / (4.0 * t.tm * t.tn));
+    if (&t == c32_tiles || c < cost) { best = &t; cost = c; }
+  }
+  return *best;
+}
+
 template <typename C2>
 static cudaError_t run_gemm(ntu_ctx* c, const GemmOp& op, int n, const void* A, const void* B, void* C) {
   GemmArgs a;
@@ -148,6 +272,17 @@ static cudaError_t run_gemm(ntu_ctx* c, const GemmOp& op, int n, const void* A, 
   a.mode = op.mode; a.pitch = op.pitch; a.krp_out = op.krp_out;
   a.rowK = op.mode ? t + op.rowK : nullptr;
   a.colK = op.mode ? t + op.colK : nullptr;
+  if (sizeof(C2) == 8 && op.mode == 0 && !op.conjA) {
+    const Cgemm32Tile& t32 = cgemm32_pick(op.M, op.N, n, c->sms);
+    const Cgemm32 fn = t32.fn[op.conjB ? 1 : 0];
+    const int bm = 8 * t32.tm, bn = 32 * t32.tn, chunks = (op.Kd + C32_BK - 1) / C32_BK;
+    const int smem = (int)sizeof(float2) * C32_BK * (bm + bn) * (chunks < C32_STAGES ? chunks : C32_STAGES);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<dim3((op.N + bn - 1) / bn, (op.M + bm - 1) / bm, n), 256, smem, c->stream>>>(
+        a, (const float2*)A, (const float2*)B, (float2*)C);
+    return after_launch(c, "k_cgemm32");
+  }
   constexpr int BM = 64, BN = 64, TM = 4, TN = 4;
   constexpr int BK = sizeof(C2) == 16 ? 8 : 16;
   dim3 grid((op.N + BN - 1) / BN, (op.M + BM - 1) / BM, n);
