@@ -1043,44 +1043,174 @@ static __device__ void als_mirror(double2* gX, int nA) {
 // eps(tau) = eps0 - sum_{lambda_i > tau lambda_max} |y_i|^2 / lambda_i,
 // y = W^H J (Eq. 4 inserted in Eq. 3); ties within 1e-14 eps0 go to the
 // larger tau.  The result is written to sm.MA (side 0) or sm.MB (side 1).
-static __device__ void als_solve(AlsShared& sm, const AlsArgs& a, int side, double2* gX,
-                                 const double2* jv, double2* pv, double2* tauv, double* dv, double* ev,
-                                 RotLog& log) {
-  const int tid = threadIdx.x, nA = a.nA;
+// The arithmetic of the implicit QR (tridiag_qr) and of its rotations is kept
+// to the last bit, as for the shifted-Cholesky solves (als_slow.cuh); one thread
+// took 8 to 11 ms a solve at n = 64 to 72 with all of it in one chain.  Now warp
+// 0 runs the sweeps on T in shared memory (both quotients of a rotation in one
+// division, the deflation test a lane per entry) while warp 1 applies the sweep
+// before to y, its real and imaginary parts in two lanes; the selection takes a
+// lane per tolerance.  What is left is the chain of a hypot and a division a
+// rotation.
+static __device__ __noinline__ void als_solve(AlsShared& sm, const AlsArgs& a, int side,
+                                              long long vitem) {
+  const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31, nA = a.nA;
+  double2* gX = a.gA + vitem * (long long)nA * nA;
+  const double2* jv = a.jv + vitem * nA;
+  double2 *pv = a.pv + vitem * nA, *tauv = a.tauv + vitem * nA;
+  RotLog log;
+  log.c = a.rc + vitem * (long long)a.rotcap;
+  log.s = a.rs + vitem * (long long)a.rotcap;
+  log.k = a.rk + vitem * (long long)a.rotcap;
+  log.cap = a.rotcap;
+  log.count = 0;
+  als_mirror(gX, nA);
+  double *d = reinterpret_cast<double*>(sm.p), *e = reinterpret_cast<double*>(sm.ap);
+  double* gain = reinterpret_cast<double*>(sm.y2);          // |y_i|^2 / lambda_i
+  int* slot = reinterpret_cast<int*>(sm.red);               // two of [log base, lo, length]
   for (int i = tid; i < nA; i += NTU_CTA) sm.y[i] = jv[i];
   __syncthreads();
-  cta_hetrd(gX, nA, dv, ev, tauv, pv, sm.red);
+  cta_hetrd(gX, nA, d, e, tauv, pv, sm.red);
   cta_apply_q(gX, nA, tauv, sm.y, true, sm.red);
-  if (tid == 0) {
-    int st = tridiag_qr(dv, ev, nA, log, sm.y);
-    if (st) sm.err |= WHY_ALS_QR;
-    double lmax = dv[0];
-    for (int i = 1; i < nA; ++i) lmax = fmax(lmax, dv[i]);
-    int kmin = a.kmin < 0 ? 0 : a.kmin, kmax = a.kmax > 20 ? 20 : a.kmax;
-    double tsel = als_tau(kmin);
-    if (lmax > 0.0 && !st) {
-      double emin = INFINITY;
-      for (int k = kmin; k <= kmax; ++k) {
-        double thr = als_tau(k) * lmax, s = 0.0;
-        for (int i = 0; i < nA; ++i)
-          if (dv[i] > thr) s += cabs2(sm.y[i]) / dv[i];
-        emin = fmin(emin, sm.eps0 - s);
+  __syncthreads();
+  if (wid == 0) {
+    const double eps = 2.220446049250313e-16;
+    int hi = nA - 1, iters = 0, base = 0, st = 0;
+    for (int t = 0;; ++t) {
+      for (int k = lid; k < hi; k += 32)
+        if (fabs(e[k]) <= eps * (fabs(d[k]) + fabs(d[k + 1]))) e[k] = 0.0;
+      __syncwarp();
+      while (hi > 0 && e[hi - 1] == 0.0) --hi;
+      int lo = hi - 1;
+      while (lo > 0 && e[lo - 1] != 0.0) --lo;
+      const int len = hi - lo;
+      if (hi > 0 && (++iters > 40 * nA || base + len > log.cap)) st = ST_NUMERIC;
+      int* sl = slot + 4 * (t & 1);
+      if (hi == 0 || st) {
+        if (lid == 0) sl[2] = 0;
+        asm volatile("bar.sync 2, 64;" ::: "memory");
+        break;
       }
-      for (int k = kmin; k <= kmax; ++k) {
-        double thr = als_tau(k) * lmax, s = 0.0;
-        for (int i = 0; i < nA; ++i)
-          if (dv[i] > thr) s += cabs2(sm.y[i]) / dv[i];
-        if (sm.eps0 - s <= emin + 1e-14 * sm.eps0) { tsel = als_tau(k); break; }
+      double *cb = log.c + base, *sb = log.s + base;
+      const double aa = d[hi - 1], b = e[hi - 1], cc = d[hi];
+      const double dl = 0.5 * (aa - cc);
+      const double den = dl + copysign(hypot(dl, b), dl);
+      const double mu = (den != 0.0) ? cc - b * b / den : cc - fabs(b);
+      double dk = d[lo], ek = e[lo], x = dk - mu, z = ek;
+      for (int k = lo; k < hi; ++k) {
+        const double r = hypot(x, z);
+        const double q = (lid == 1 ? -z : x) / r;
+        double c = __shfl_sync(0xffffffffu, q, 0), s = __shfl_sync(0xffffffffu, q, 1);
+        if (r == 0.0) { c = 1.0; s = 0.0; }
+        const double dk1 = d[k + 1], cs = c * s;
+        const double nk = c * c * dk - 2.0 * cs * ek + s * s * dk1;
+        const double nk1 = s * s * dk + 2.0 * cs * ek + c * c * dk1;
+        const double ne = cs * (dk - dk1) + (c * c - s * s) * ek;
+        if (lid == 0) {
+          if (k > lo) e[k - 1] = r;
+          d[k] = nk;
+          cb[k - lo] = c;
+          sb[k - lo] = s;
+        }
+        x = ne;
+        dk = nk1;
+        if (k + 1 < hi) {
+          const double ek1 = e[k + 1];
+          z = -s * ek1;
+          ek = c * ek1;
+        }
       }
-      double thr = tsel * lmax;
-      for (int i = 0; i < nA; ++i)
-        sm.y[i] = dv[i] > thr ? cscale(sm.y[i], 1.0 / dv[i]) : cz();
-      rotlog_apply_z(log, sm.y);
-    } else {
-      for (int i = 0; i < nA; ++i) sm.y[i] = cz();
+      __syncwarp();
+      if (lid == 0) {
+        d[hi] = dk;
+        e[hi - 1] = x;
+        sl[0] = base; sl[1] = lo; sl[2] = len;
+      }
+      for (int i = lid; i < len; i += 32) log.k[base + i] = lo + i;
+      base += len;
+      asm volatile("bar.sync 2, 64;" ::: "memory");
     }
-    sm.tau_sel = tsel;
-    sm.n_eig += 1;
+    if (lid == 0) {
+      slot[8] = base;
+      slot[9] = st;
+    }
+  } else if (wid == 1) {
+    for (int t = 0;; ++t) {
+      asm volatile("bar.sync 2, 64;" ::: "memory");
+      const int* sl = slot + 4 * (t & 1);
+      const int base = sl[0], lo = sl[1], len = sl[2];
+      if (len == 0) break;
+      if (lid < 2) {
+        double* yc = reinterpret_cast<double*>(sm.y) + lid;
+        double yk = yc[2 * lo];
+#pragma unroll 4
+        for (int i = 0; i < len; ++i) {
+          const double c = log.c[base + i], s = log.s[base + i], yk1 = yc[2 * (lo + i + 1)];
+          yc[2 * (lo + i)] = c * yk - s * yk1;
+          yk = s * yk + c * yk1;
+        }
+        yc[2 * (lo + len)] = yk;
+      }
+    }
+  }
+  __syncthreads();
+  const int count = slot[8], st = slot[9];
+  for (int i = tid; i < nA; i += NTU_CTA) gain[i] = cabs2(sm.y[i]) / d[i];
+  __syncthreads();
+  if (wid == 0) {
+    double lmax = d[0];
+    for (int i = lid; i < nA; i += 32) lmax = fmax(lmax, d[i]);
+    lmax = warp_max(lmax);
+    const int kmin = a.kmin < 0 ? 0 : a.kmin, kmax = a.kmax > 20 ? 20 : a.kmax;
+    double tsel = als_tau(kmin), thr = INFINITY;
+    if (lmax > 0.0 && !st) {
+      const int k = kmin + lid;
+      double eps = INFINITY;
+      if (k <= kmax) {
+        const double lim = als_tau(k) * lmax;
+        double s = 0.0;
+        for (int i = 0; i < nA; ++i)
+          if (d[i] > lim) s += gain[i];
+        eps = sm.eps0 - s;
+      }
+      const double emin = -warp_max(-eps);
+      const unsigned in = __ballot_sync(0xffffffffu, k <= kmax && eps <= emin + 1e-14 * sm.eps0);
+      if (in) tsel = als_tau(kmin + __ffs(in) - 1);
+      thr = tsel * lmax;
+    }
+    if (lid == 0) {
+      if (st) sm.err |= WHY_ALS_QR;
+      sm.tau_sel = tsel;
+      sm.n_eig += 1;
+      sm.red[8] = thr;                                      // past the slots
+    }
+  }
+  __syncthreads();
+  const double thr = sm.red[8];
+  for (int i = tid; i < nA; i += NTU_CTA) {
+    const double lam = d[i];
+    sm.y[i] = lam > thr ? cscale(sm.y[i], 1.0 / lam) : cz();
+  }
+  __syncthreads();
+  if (wid == 0) {
+    // y <- Z y: the rotations in reverse, 32 of them loaded at a time
+    double* yc = reinterpret_cast<double*>(sm.y) + (lid & 1);
+    for (int top = count; top > 0; top -= 32) {
+      const int t = top - 1 - lid;
+      const double cl = t >= 0 ? log.c[t] : 1.0, sl = t >= 0 ? log.s[t] : 0.0;
+      const int kl = t >= 0 ? log.k[t] : 0;
+      const int m = top < 32 ? top : 32;
+      for (int i = 0; i < m; ++i) {
+        const double c = __shfl_sync(0xffffffffu, cl, i), s = __shfl_sync(0xffffffffu, sl, i);
+        const int k = __shfl_sync(0xffffffffu, kl, i);
+        const double u = yc[2 * k], v = yc[2 * k + 2];
+        __syncwarp();
+        if (lid < 2) {
+          yc[2 * k] = c * u + s * v;
+          yc[2 * k + 2] = -s * u + c * v;
+        }
+        __syncwarp();
+      }
+    }
   }
   __syncthreads();
   cta_apply_q(gX, nA, tauv, sm.y, false, sm.red);
@@ -1229,8 +1359,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
           if (nA <= LOW_SH_MAX) als_solve_spectrum<true>(sm, a, side, gX, jv, pv, tauv, dv, ev, Tm, log);
           else als_solve_spectrum<false>(sm, a, side, gX, jv, pv, tauv, dv, ev, Tm, log);
         } else {
-          als_mirror(gX, nA);
-          als_solve(sm, a, side, gX, jv, pv, tauv, dv, ev, log);
+          als_solve(sm, a, side, vitem);
         }
       }
     }
