@@ -1241,6 +1241,9 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
   const long long item = SPLIT ? blockIdx.x / split : blockIdx.x, vitem = blockIdx.x;
   const int K = a.K, D = a.D, ng = a.ng, nA = a.nA;
   const double2* g = a.g + item * (long long)ng * ng;
+  // no metric: the identity (the simple update, FP64): each of its two products
+  // would take one SM 0.09 ms at K = 16
+  const bool ident = F64 && a.g == nullptr;
   const double2* RA = a.RA + item * K * K;
   const double2* RB = a.RB + item * K * K;
   double2* x0 = a.x0 + vitem * ng;
@@ -1308,8 +1311,12 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
     for (int r = wid; r < ng; r += NTU_WARPS) {
       const double2* gr = g + (size_t)r * ng;
       double2 acc = cz();
-      for (int c = lid; c < ng; c += 32) acc = cfma(gr[c], x0[c], acc);
-      acc = warp_sum2(acc);
+      if (ident) {
+        acc = x0[r];
+      } else {
+        for (int c = lid; c < ng; c += 32) acc = cfma(gr[c], x0[c], acc);
+        acc = warp_sum2(acc);
+      }
       if (lid == 0) {
         gx0[r] = acc;
         e0 += cmulc(x0[r], acc).x;
@@ -1398,8 +1405,12 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
     for (int r = wid; r < ng; r += NTU_WARPS) {
       const double2* gr = g + (size_t)r * ng;
       double2 acc = cz();
-      for (int c = lid; c < ng; c += 32) acc = cfma(gr[c], xv[c], acc);
-      acc = warp_sum2(acc);
+      if (ident) {
+        acc = xv[r];
+      } else {
+        for (int c = lid; c < ng; c += 32) acc = cfma(gr[c], xv[c], acc);
+        acc = warp_sum2(acc);
+      }
       if (lid == 0) eps += cmulc(xv[r], acc).x;
     }
   }

@@ -40,7 +40,8 @@ static_assert(OZ_SMEM_BYTES + 1023 <= sizeof(SvdSmem) + ALS_OZ_SLACK,
 
 struct AlsArgs {
   int D, K, ng, nA, sweeps, kmin, kmax;
-  const double2* g; const double2* RA; const double2* RB;
+  const double2* g;            // NULL: the identity (FP64 contexts, no sweeps)
+  const double2* RA; const double2* RB;
   double2* MA; double2* MB; double* info;
   int* path_counts;            // [Gershgorin+CG, shifted Cholesky, eigen] solves (may be NULL)
   double2 *x0, *gx0, *Tm, *gA, *gC, *jv, *pv, *tauv;

@@ -644,8 +644,9 @@ static int su_bond(ntu_ctx* c, int bond, const double2* gate_dev, double* info_d
   CK(launch_orient(c, bond, W.cA2, W.cB2, W.cTa, W.cTb), "orient");
   CK(launch_gate_qr(c, 1, W.cTa, W.cTb, gate_dev, bond >= 2 ? 1 : 0, W.QA, W.RA, W.QB, W.RB),
      "gate + QR");
-  CK(launch_identity_metric(c, W.g), "identity metric");
-  CK(launch_als(c, 1, W.g, W.RA, W.RB, W.MA, W.MB, info_dev, 0), "SU truncation");
+  const bool f64 = c->cfg.precision == NTU_FP64;         // there the identity needs no array
+  if (!f64) CK(launch_identity_metric(c, W.g), "identity metric");
+  CK(launch_als(c, 1, f64 ? nullptr : W.g, W.RA, W.RB, W.MA, W.MB, info_dev, 0), "SU truncation");
   CK(launch_recompose(c, 1, W.QA, W.QB, W.MA, W.MB, W.cA2, W.cB2), "recompose");
   CK(launch_deorient(c, bond, W.cA2, W.cB2, W.A, W.B), "write back");
   CK(launch_su_weight(c, bond, 1, 1, W.A, W.B, W.A, W.B), "SU unweight");

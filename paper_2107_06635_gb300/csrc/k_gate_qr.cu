@@ -1,7 +1,9 @@
 // Gate split, gate application and QR reduction (Fig. 2(a,b)), recomposition
 // of the updated site tensors (Fig. 2(e)), lattice orientation of the four
 // bonds, single-site Trotter gates and the cluster estimator.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+#include <string.h>
 
 #include "ntu_dev.cuh"
 #include "ntu_impl.h"
@@ -333,8 +335,169 @@ __global__ void __launch_bounds__(NTU_CTA) k_qr(int m, int K, double2* __restric
   }
 }
 
+// The same factorisation on a cluster of CL CTAs, for the FP64 contexts with
+// few matrices: one SM's FP64 pipe took 0.94 ms at m = 1024, K = 16.  Each CTA
+// holds a run of rows; the norm (each CTA's largest entry and its sum of
+// squares relative to that) and the inner products with the later columns go
+// to every CTA's shared memory and are added there in the order of the ranks,
+// so all CTAs go on with the same numbers: two cluster barriers a reflector, one
+// a column of Q.  Two buffers per exchange, by its number: a CTA can be one
+// barrier ahead of another's reads, never two.
+constexpr int CL = 8;                                    // the portable cluster size
+struct QrHead { double mx, s2; double2 alpha; };         // a CTA's part of a column's norm
+__global__ void __launch_bounds__(NTU_CTA) k_qr_cluster(int m, int K, double2* __restrict__ Mg,
+                                                        double2* __restrict__ Qcm,
+                                                        double2* __restrict__ QA, double2* __restrict__ RA,
+                                                        double2* __restrict__ QB, double2* __restrict__ RB,
+                                                        int* paths) {
+  __shared__ double2 taus[32];
+  __shared__ double betas[32];
+  __shared__ double sred[2 * NTU_WARPS];
+  __shared__ QrHead head[2][CL];
+  __shared__ double2 dots[2][CL][32];
+  __shared__ double2 f[32];
+  __shared__ double sc[8];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), item = blockIdx.x / CL, side = blockIdx.y, tid = threadIdx.x;
+  const int wid = tid >> 5, lid = tid & 31;
+  if (tid == 0 && rank == 0 && paths) atomicAdd(paths + 7, 1);
+  cl.sync();                                             // every CTA is there to be written to
+  double2* M = Mg + ((size_t)item * 2 + side) * m * K;
+  double2* Qc = Qcm + ((size_t)item * 2 + side) * m * K;
+  const int run = (m + CL - 1) / CL, r0 = min(rank * run, m), r1 = min(r0 + run, m);
+  int ex = 0;                                            // number of the exchange of inner products
+  // f[c] = w sum conj(v) X[:, c] for columns c0 <= c < K, over all rows >= j
+  auto project = [&](const double2* v, const double2* X, int j, int c0, double2 w) {
+    for (int c = c0 + wid; c < K; c += NTU_WARPS) {
+      const double2* x = X + (size_t)c * m;
+      double2 dot = cz();
+      for (int i = max(r0, j) + lid; i < r1; i += 32) dot = cfmac(v[i], x[i], dot);
+      dot = warp_sum2(dot);
+      if (lid < CL) *cl.map_shared_rank(&dots[ex & 1][rank][c], lid) = dot;
+    }
+    cl.sync();
+    if (tid >= c0 && tid < K) {
+      double2 t = dots[ex & 1][0][tid];
+      for (int q = 1; q < CL; ++q) t = cadd(t, dots[ex & 1][q][tid]);
+      f[tid] = cmul(w, t);
+    }
+    ++ex;
+    __syncthreads();
+  };
+  for (int j = 0; j < K; ++j) {
+    double2* col = M + (size_t)j * m;
+    const int i0 = max(r0, j + 1);
+    double mx = 0.0, xs2 = 0.0;
+    for (int i = i0 + tid; i < r1; i += NTU_CTA) mx = fmax(mx, fmax(fabs(col[i].x), fabs(col[i].y)));
+    mx = block_max(mx, sred);
+    if (mx > 0.0) {
+      const double inv = 1.0 / mx;
+      for (int i = i0 + tid; i < r1; i += NTU_CTA) xs2 += cabs2(cscale(col[i], inv));
+    }
+    xs2 = block_sum(xs2, sred);
+    if (tid < CL) {
+      const bool own = j >= r0 && j < r1;
+      const double2 al = own ? col[j] : cz();
+      *cl.map_shared_rank(&head[j & 1][rank], tid) = QrHead{mx, xs2, al};
+    }
+    cl.sync();
+    if (tid == 0) {
+      double2 alpha = cz();
+      double big = 0.0, s2 = 0.0;
+      for (int q = 0; q < CL; ++q) {
+        const QrHead h = head[j & 1][q];
+        big = fmax(big, h.mx);
+        alpha = cadd(alpha, h.alpha);                    // one of them has the row
+      }
+      double2 tau = cz(), scale = make_double2(1.0, 0.0);
+      double beta = alpha.x;
+      if (!(big == 0.0 && alpha.y == 0.0)) {
+        const double amax = fmax(big, fmax(fabs(alpha.x), fabs(alpha.y))), inv = 1.0 / amax;
+        for (int q = 0; q < CL; ++q) {
+          const QrHead h = head[j & 1][q];
+          const double t = h.mx * inv;
+          if (h.mx > 0.0) s2 = fma(h.s2, t * t, s2);
+        }
+        const double nrm = amax * sqrt(cabs2(cscale(alpha, inv)) + s2);
+        beta = alpha.x >= 0.0 ? -nrm : nrm;
+        tau = make_double2((beta - alpha.x) / beta, -alpha.y / beta);
+        scale = cdiv(make_double2(1.0, 0.0), make_double2(alpha.x - beta, alpha.y));
+      }
+      taus[j] = tau;
+      betas[j] = beta;
+      sc[0] = scale.x;
+      sc[1] = scale.y;
+    }
+    __syncthreads();
+    const double2 tau = taus[j], scale = make_double2(sc[0], sc[1]);
+    for (int i = i0 + tid; i < r1; i += NTU_CTA) col[i] = cmul(col[i], scale);
+    if (tid == 0 && j >= r0 && j < r1) col[j] = make_double2(1.0, 0.0);
+    __syncthreads();
+    if ((tau.x != 0.0 || tau.y != 0.0) && j + 1 < K) {
+      project(col, M, j, j + 1, cconj(tau));
+      for (int c = j + 1 + wid; c < K; c += NTU_WARPS) {
+        double2* x = M + (size_t)c * m;
+        const double2 fc = f[c];
+        for (int i = max(r0, j) + lid; i < r1; i += 32) x[i] = cfms(fc, col[i], x[i]);
+      }
+      __syncthreads();
+    }
+  }
+  // Q = H_0 ... H_{K-1} [I; 0]
+  for (int c = wid; c < K; c += NTU_WARPS)
+    for (int i = r0 + lid; i < r1; i += 32) Qc[(size_t)c * m + i] = make_double2(i == c ? 1.0 : 0.0, 0.0);
+  __syncthreads();
+  for (int j = K - 1; j >= 0; --j) {
+    const double2 tau = taus[j];
+    if (tau.x == 0.0 && tau.y == 0.0) continue;
+    const double2* v = M + (size_t)j * m;
+    project(v, Qc, j, j, tau);
+    for (int c = j + wid; c < K; c += NTU_WARPS) {
+      double2* x = Qc + (size_t)c * m;
+      const double2 fc = f[c];
+      for (int i = max(r0, j) + lid; i < r1; i += 32) x[i] = cfms(fc, v[i], x[i]);
+    }
+    __syncthreads();
+  }
+  double2* Qo = (side ? QB : QA) + (size_t)item * m * K;
+  double2* Ro = (side ? RB : RA) + (size_t)item * K * K;
+  for (int idx = tid; idx < (r1 - r0) * K; idx += NTU_CTA) {
+    const int i = r0 + idx / K, c = idx % K;
+    const double2 q = Qc[(size_t)c * m + i];
+    Qo[(size_t)i * K + c] = betas[c] < 0.0 ? make_double2(-q.x, -q.y) : q;
+  }
+  const int k1 = min(r1, K);
+  for (int idx = tid; r0 < k1 && idx < (k1 - r0) * K; idx += NTU_CTA) {
+    const int j = r0 + idx / K, c = idx % K;
+    const double2 v = c > j ? M[(size_t)c * m + j] : (c == j ? make_double2(betas[j], 0.0) : cz());
+    Ro[j * K + c] = betas[j] < 0.0 ? make_double2(-v.x, -v.y) : v;
+  }
+}
+
+// Launches a kernel of CTAs in clusters of CL.
+template <typename... P, typename... A>
+static cudaError_t launch_clusters(void (*kern)(P...), dim3 grid, cudaStream_t stream, A... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(NTU_CTA, 1, 1);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 // ------------------------------------------------------------ recompose
 // T' = Q M (Fig. 2(e)) put back into [p, l, u, r, dn] and normalised.
+// SPREAD: an item and side on a cluster (FP64 contexts with few items; 0.15 ms
+// on one SM at D = 8), the squared norm added over the CTAs.
+template <bool SPREAD>
 __global__ void __launch_bounds__(NTU_CTA) k_recompose(int dp, int D, int K,
                                                        const double2* __restrict__ QA,
                                                        const double2* __restrict__ QB,
@@ -345,7 +508,9 @@ __global__ void __launch_bounds__(NTU_CTA) k_recompose(int dp, int D, int K,
   __shared__ double2 Ms[32 * 8];
   __shared__ float4 Mdf[32 * 8];
   __shared__ double sred[2 * NTU_WARPS];
-  const int item = blockIdx.x, side = blockIdx.y, tid = threadIdx.x;
+  __shared__ double part[CL];
+  const int item = SPREAD ? blockIdx.x / CL : blockIdx.x, side = blockIdx.y, tid = threadIdx.x;
+  const int rank = SPREAD ? blockIdx.x % CL : 0, step = SPREAD ? CL * NTU_CTA : NTU_CTA;
   const int D2 = D * D, D3 = D2 * D, D4 = D3 * D, m = dp * D3;
   const double2* Q = (side ? QB : QA) + (size_t)item * m * K;
   const double2* Mx = (side ? MB : MA) + (size_t)item * K * D;
@@ -379,7 +544,7 @@ __global__ void __launch_bounds__(NTU_CTA) k_recompose(int dp, int D, int K,
         }
     }
   } else
-  for (int idx = tid; idx < m * D; idx += NTU_CTA) {
+  for (int idx = rank * NTU_CTA + tid; idx < m * D; idx += step) {
     int row = idx / D, a = idx % D;
     double2 acc = cz();
     for (int k = 0; k < K; ++k) acc = cfma(Q[(size_t)row * K + k], Ms[k * D + a], acc);
@@ -390,10 +555,19 @@ __global__ void __launch_bounds__(NTU_CTA) k_recompose(int dp, int D, int K,
     out[(size_t)p * D4 + l * D3 + u * D2 + rr * D + n_] = acc;
     nrm2 += cabs2(acc);
   }
-  double nrm = sqrt(block_sum(nrm2, sred));
+  nrm2 = block_sum(nrm2, sred);
+  if (SPREAD) {
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    cl.sync();                                           // every CTA is there to be written to
+    if (tid < CL) *cl.map_shared_rank(&part[rank], tid) = nrm2;
+    cl.sync();                                           // orders the CTAs' writes of out too
+    nrm2 = part[0];
+    for (int q = 1; q < CL; ++q) nrm2 += part[q];
+  }
+  double nrm = sqrt(nrm2);
   double sc = nrm > 0.0 ? 1.0 / nrm : 1.0;
   __syncthreads();
-  for (int idx = tid; idx < dp * D4; idx += NTU_CTA) out[idx] = cscale(out[idx], sc);
+  for (int idx = rank * NTU_CTA + tid; idx < dp * D4; idx += step) out[idx] = cscale(out[idx], sc);
 }
 
 // ------------------------------------------------------------ orientation
@@ -477,13 +651,19 @@ __global__ void __launch_bounds__(NTU_CTA) k_measure(int d, int danc, int D,
                                                      double2* __restrict__ out) {
   __shared__ double sred[2 * NTU_WARPS];
   const int tid = threadIdx.x;
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const int first = (int)cl.block_rank() * NTU_CTA + tid, step = CL * NTU_CTA;
   const int dp = d * danc, D2 = D * D, D3 = D2 * D, D4 = D3 * D;
-  // leaf edge tensors: El keeps r, Eu keeps dn, Er keeps l, Ed keeps u
-  for (int idx = tid; idx < 4 * D2; idx += NTU_CTA) {
+  // leaf edge tensors: El keeps r, Eu keeps dn, Er keeps l, Ed keeps u; 32
+  // entries a CTA, a warp for each value of the first summed leg
+  __shared__ double2 pe[NTU_WARPS][32];
+  const int wid = tid >> 5, lid = tid & 31;
+  for (int i0 = (int)cl.block_rank(); i0 < 4 * D2; i0 += 32 * CL) {
+    const int idx = i0 + lid * CL;
     int which = idx / D2, x = (idx % D2) / D, y = idx % D;
     double2 acc = cz();
-    for (int p = 0; p < dp; ++p)
-      for (int a = 0; a < D; ++a)
+    for (int p = 0; p < dp && idx < 4 * D2; ++p)
+      for (int a = wid; a < D; a += NTU_WARPS)
         for (int b = 0; b < D; ++b)
           for (int c = 0; c < D; ++c) {
             size_t ix, iy, base = (size_t)p * D4;
@@ -493,9 +673,15 @@ __global__ void __launch_bounds__(NTU_CTA) k_measure(int d, int danc, int D,
             else { ix = base + a * D3 + x * D2 + b * D + c; iy = base + a * D3 + y * D2 + b * D + c; }
             acc = cfma(N[ix], cconj(N[iy]), acc);
           }
-    E[idx] = acc;
+    pe[wid][lid] = acc;
+    __syncthreads();
+    if (wid == 0 && idx < 4 * D2) {
+      for (int q = 1; q < NTU_WARPS; ++q) acc = cadd(acc, pe[q][lid]);
+      E[idx] = acc;
+    }
+    __syncthreads();
   }
-  __syncthreads();
+  cl.sync();
   // contract the four legs of T one at a time: S <- sum_leg S * E_leg[leg, leg']
   const double2* src = T;
   double2* bufs[2] = {S1, S2};
@@ -503,16 +689,17 @@ __global__ void __launch_bounds__(NTU_CTA) k_measure(int d, int danc, int D,
     double2* dst = bufs[leg & 1];
     const double2* El = E + leg * D2;      // leg 0: l uses El (keeps r), 1: u/Eu, 2: r/Er, 3: dn/Ed
     int stride = leg == 0 ? D3 : leg == 1 ? D2 : leg == 2 ? D : 1;
-    for (int idx = tid; idx < dp * D4; idx += NTU_CTA) {
+    for (int idx = first; idx < dp * D4; idx += step) {
       int a = (idx / stride) % D;
       int base = idx - a * stride;
       double2 acc = cz();
       for (int x = 0; x < D; ++x) acc = cfma(src[base + x * stride], El[x * D + a], acc);
       dst[idx] = acc;
     }
-    __syncthreads();
+    cl.sync();
     src = dst;
   }
+  if (cl.block_rank() != 0) return;
   // num = sum conj(T[q..]) O_full[q, p] V[p..]; den = sum conj(T[p..]) V[p..]
   double2 num = cz(), den = cz();
   for (int idx = tid; idx < dp * D4; idx += NTU_CTA) {
@@ -546,6 +733,12 @@ static inline int grid_for(long long work) {
   return (int)(b < 1 ? 1 : (b > 65535 ? 65535 : b));
 }
 
+// The FP64 contexts' QR and recomposition on clusters: where every item and side
+// has one at the same time, and the rows are worth the barriers (two a column).
+static bool spread_items(const ntu_ctx* c, int n) {
+  return c->cfg.precision == NTU_FP64 && (long long)n * 2 * CL <= c->sms && c->plan.m >= 128;
+}
+
 cudaError_t launch_gate_qr(ntu_ctx* c, int n, const double2* Ta, const double2* Tb,
                            const double2* G, int swap_sites, double2* QA, double2* RA,
                            double2* QB, double2* RB) {
@@ -572,6 +765,12 @@ cudaError_t launch_gate_qr(ntu_ctx* c, int n, const double2* Ta, const double2* 
                                                  c->d_paths);
     return after_launch(c, "k_qr");
   }
+  if (spread_items(c, n)) {
+    e = launch_clusters(k_qr_cluster, dim3(n * CL, 2), c->stream, P.m, P.K, W.Mg, W.Qcm, QA, RA, QB, RB,
+                        c->d_paths);
+    if (e != cudaSuccess) return e;
+    return after_launch(c, "k_qr_cluster");
+  }
   k_qr<<<dim3(n, 2), NTU_CTA, 0, c->stream>>>(P.m, P.K, W.Mg, W.Qcm, QA, RA, QB, RB, nullptr,
                                                c->d_paths);
   return after_launch(c, "k_qr");
@@ -581,7 +780,13 @@ cudaError_t launch_recompose(ntu_ctx* c, int n, const double2* QA, const double2
                              const double2* MA, const double2* MB, double2* Ta_out,
                              double2* Tb_out) {
   const Plan& P = c->plan;
-  k_recompose<<<dim3(n, 2), NTU_CTA, 0, c->stream>>>(P.dp, P.D, P.K, QA, QB, MA, MB, Ta_out,
+  if (spread_items(c, n)) {
+    cudaError_t e = launch_clusters(k_recompose<true>, dim3(n * CL, 2), c->stream, P.dp, P.D, P.K, QA, QB,
+                                    MA, MB, Ta_out, Tb_out, 0);
+    if (e != cudaSuccess) return e;
+    return after_launch(c, "k_recompose");
+  }
+  k_recompose<false><<<dim3(n, 2), NTU_CTA, 0, c->stream>>>(P.dp, P.D, P.K, QA, QB, MA, MB, Ta_out,
                                                      Tb_out, c->cfg.precision != NTU_FP64);
   return after_launch(c, "k_recompose");
 }
@@ -610,8 +815,9 @@ cudaError_t launch_measure(ntu_ctx* c, const double2* T, const double2* N, const
                            double2* out) {
   const Plan& P = c->plan;
   Work& W = c->w;
-  k_measure<<<1, NTU_CTA, 0, c->stream>>>(P.d, P.d_anc, P.D, T, N, op, W.mscr1, W.mscr2,
-                                          W.medge, out);
+  cudaError_t e = launch_clusters(k_measure, dim3(CL), c->stream, P.d, P.d_anc, P.D, T, N, op,
+                                  W.mscr1, W.mscr2, W.medge, out);
+  if (e != cudaSuccess) return e;
   return after_launch(c, "k_measure");
 }
 
