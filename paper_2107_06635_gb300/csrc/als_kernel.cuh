@@ -345,6 +345,7 @@ static __device__ int als_tilt_fast(AlsShared& sm, const AlsArgs& a, int mode) {
 // when min R_qq <= 1e-12 max R_qq (the SVD tilt then handles the nearly
 // rank-deficient factor).  Gram-Schmidt takes D dependent reductions where
 // the one-sided Jacobi SVD takes some 15 rounds of FP64 rotations.
+template <bool F64>
 static __device__ int als_tilt_qr(AlsShared& sm, const AlsArgs& a, int side) {
   const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31, K = a.K, D = a.D;
   double2* Y = side == 0 ? sm.MB : sm.MA;
@@ -366,52 +367,100 @@ static __device__ int als_tilt_qr(AlsShared& sm, const AlsArgs& a, int side) {
     if (lid == 0) n2[q] = s2;
   }
   __syncthreads();
-  for (int q = 0; q < D; ++q) {
-    // project out the previous columns; a second pass only when the first
-    // left less than 1/sqrt(2) of the norm (the DGKS criterion: then the
-    // column is orthogonal to working precision)
-    double before = n2[q];
-    for (int pass = 0; pass < 2 && q > 0; ++pass) {
-      // c_p = Q_p^H v for p < q (warp p), then v -= sum_p Q_p c_p
-      for (int p = wid; p < q; p += NTU_WARPS) {
-        double2 c = lid < K ? cmulc(Q[p * 32 + lid], Q[q * 32 + lid]) : cz();
-        c = warp_sum2(c);
-        if (lid == 0) {
-          sm.ph[p] = c;
-          R[p * 32 + q] = cadd(R[p * 32 + q], c);
+  if constexpr (F64) {
+    double lo = INFINITY, hi = 0.0;                       // of the R_qq (warp 0)
+    for (int q = 0; q < D; ++q) {
+      // as below, warp 0 taking the column from its projections to its scaling
+      // (two barriers a pass; see block_sum)
+      for (int pass = 0; pass < 2; ++pass) {
+        // c_p = Q_p^H v for p < q (warp p)
+        for (int p = wid; p < q; p += NTU_WARPS) {
+          double2 c = lid < K ? cmulc(Q[p * 32 + lid], Q[q * 32 + lid]) : cz();
+          c = warp_sum2(c);
+          if (lid == 0) {
+            sm.ph[p] = c;
+            R[p * 32 + q] = cadd(R[p * 32 + q], c);
+          }
         }
+        if (q > 0) __syncthreads();
+        if (wid == 0) {
+          // v -= sum_p Q_p c_p, then Q_q = v / |v|
+          double2 v = lid < K ? Q[q * 32 + lid] : cz();
+          double s2 = n2[q];
+          bool again = false;
+          if (q > 0) {
+            const double before = s2;
+            if (lid < K)
+              for (int p = 0; p < q; ++p) v = cfms(Q[p * 32 + lid], sm.ph[p], v);
+            s2 = warp_sum(lid < K ? cabs2(v) : 0.0);
+            again = pass == 0 && !(s2 >= 0.5 * before);
+          }
+          if (!again) {
+            const double rq = sqrt(s2);
+            v = rq > 0.0 ? cscale(v, 1.0 / rq) : cz();
+            lo = q == 0 || rq < lo ? rq : lo;
+            hi = q == 0 || rq > hi ? rq : hi;
+            if (lid == 0) R[q * 32 + q] = make_double2(rq, 0.0);
+          }
+          if (lid < K) Q[q * 32 + lid] = v;
+          if (lid == 0) {
+            n2[q] = s2;
+            sm.flag = again ? 1 : (lo > 1e-12 * hi && isfinite(hi) ? 2 : 0);
+          }
+        }
+        __syncthreads();
+        if (sm.flag != 1) break;
       }
-      __syncthreads();
-      if (tid < K) {
-        double2 v = Q[q * 32 + tid];
-        for (int p = 0; p < q; ++p) v = cfms(Q[p * 32 + tid], sm.ph[p], v);
-        Q[q * 32 + tid] = v;
-      }
-      __syncthreads();
-      if (wid == 0) {
-        double s2 = lid < K ? cabs2(Q[q * 32 + lid]) : 0.0;
-        s2 = warp_sum(s2);
-        if (lid == 0) n2[q] = s2;
-      }
-      __syncthreads();
-      const double after = n2[q];
-      if (after >= 0.5 * before) break;
-      before = after;
     }
-    const double rq = sqrt(n2[q]);
-    if (tid < K) Q[q * 32 + tid] = rq > 0.0 ? cscale(Q[q * 32 + tid], 1.0 / rq) : cz();
-    if (tid == 0) {
-      R[q * 32 + q] = make_double2(rq, 0.0);
-      rd[q] = rq;
+    if (sm.flag == 0) return 0;
+  } else {
+    for (int q = 0; q < D; ++q) {
+      // project out the previous columns; a second pass only when the first
+      // left less than 1/sqrt(2) of the norm (the DGKS criterion: then the
+      // column is orthogonal to working precision)
+      double before = n2[q];
+      for (int pass = 0; pass < 2 && q > 0; ++pass) {
+        // c_p = Q_p^H v for p < q (warp p), then v -= sum_p Q_p c_p
+        for (int p = wid; p < q; p += NTU_WARPS) {
+          double2 c = lid < K ? cmulc(Q[p * 32 + lid], Q[q * 32 + lid]) : cz();
+          c = warp_sum2(c);
+          if (lid == 0) {
+            sm.ph[p] = c;
+            R[p * 32 + q] = cadd(R[p * 32 + q], c);
+          }
+        }
+        __syncthreads();
+        if (tid < K) {
+          double2 v = Q[q * 32 + tid];
+          for (int p = 0; p < q; ++p) v = cfms(Q[p * 32 + tid], sm.ph[p], v);
+          Q[q * 32 + tid] = v;
+        }
+        __syncthreads();
+        if (wid == 0) {
+          double s2 = lid < K ? cabs2(Q[q * 32 + lid]) : 0.0;
+          s2 = warp_sum(s2);
+          if (lid == 0) n2[q] = s2;
+        }
+        __syncthreads();
+        const double after = n2[q];
+        if (after >= 0.5 * before) break;
+        before = after;
+      }
+      const double rq = sqrt(n2[q]);
+      if (tid < K) Q[q * 32 + tid] = rq > 0.0 ? cscale(Q[q * 32 + tid], 1.0 / rq) : cz();
+      if (tid == 0) {
+        R[q * 32 + q] = make_double2(rq, 0.0);
+        rd[q] = rq;
+      }
+      __syncthreads();
     }
-    __syncthreads();
+    double lo = rd[0], hi = rd[0];
+    for (int q = 1; q < D; ++q) {
+      lo = rd[q] < lo ? rd[q] : lo;
+      hi = rd[q] > hi ? rd[q] : hi;
+    }
+    if (!(lo > 1e-12 * hi) || !isfinite(hi)) return 0;
   }
-  double lo = rd[0], hi = rd[0];
-  for (int q = 1; q < D; ++q) {
-    lo = rd[q] < lo ? rd[q] : lo;
-    hi = rd[q] > hi ? rd[q] : hi;
-  }
-  if (!(lo > 1e-12 * hi) || !isfinite(hi)) return 0;
   // Z R^T into W, then both factors in place
   for (int idx = tid; idx < K * D; idx += NTU_CTA) {
     const int i = idx / D, q = idx % D;
@@ -918,8 +967,8 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
       ghi = fmax(ghi, d + sgi);
     }
   }
-  glo = block_min(glo, sm.red);
-  const double bmax = block_max(ghi, sm.red);               // >= lambda_max
+  glo = block_min<F64>(glo, sm.red);
+  const double bmax = block_max<F64>(ghi, sm.red);               // >= lambda_max
   if (!(bmax > 0.0) || !isfinite(bmax) || !isfinite(glo)) return 0;
   const double sigma = (tau_max + 1e-12) * bmax;
   if (glo > sigma) {
@@ -943,8 +992,8 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
       js += cabs2(jv[i]);
       rs += cabs2(r);
     }
-    js = block_sum(js, sm.red);
-    rs = block_sum(rs, sm.red);
+    js = block_sum<F64>(js, sm.red);
+    rs = block_sum<F64>(rs, sm.red);
     const double stop = (df ? 1e-28 : 1e-30) * js;          // |r| <= 1e-14 (1e-15) |J|
     const double floor2 = (df ? 1e-24 : 1e-26) * js;        // rounding floor of the recursion
     const double accept = 1e-26 * js;                       // FP64 residual <= 1e-13 |J|
@@ -961,7 +1010,7 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
           sm.y2[i] = r; sm.p[i] = r;
           r64 += cabs2(r);
         }
-        r64 = block_sum(r64, sm.red);
+        r64 = block_sum<F64>(r64, sm.red);
         if (r64 <= accept) { conv = 1; break; }
         if (++checks > 3) break;
         rs = r64; prev = r64; small = false;
@@ -970,7 +1019,7 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
       als_matvec(sm, gX, gXdf, sm.p, sm.ap, nA, df);
       double pap = 0.0;
       for (int i = tid; i < nA; i += NTU_CTA) pap += cmulc(sm.p[i], sm.ap[i]).x;
-      pap = block_sum(pap, sm.red);
+      pap = block_sum<F64>(pap, sm.red);
       if (!(pap > 0.0)) break;
       const double alpha = rs / pap;
       double rn = 0.0;
@@ -981,7 +1030,7 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
         sm.y[i] = x; sm.y2[i] = r;
         rn += cabs2(r);
       }
-      rn = block_sum(rn, sm.red);
+      rn = block_sum<F64>(rn, sm.red);
       // converged, or stalled at the rounding floor of the recursion
       small = rn <= stop || (it >= 2 && rn > 0.25 * prev && rn <= floor2);
       prev = rn;
@@ -1333,7 +1382,7 @@ __global__ void __launch_bounds__(NTU_CTA, MINB) k_als(AlsArgs a) {
   bool tc_dead = false;
   for (int s = 0; s < a.sweeps && !tc_dead; ++s) {
     for (int side = 0; side < 2; ++side) {
-      if ((s > 0 || side > 0) && !als_tilt_qr(sm, a, side) && !als_tilt_fast(sm, a, side))
+      if ((s > 0 || side > 0) && !als_tilt_qr<F64>(sm, a, side) && !als_tilt_fast(sm, a, side))
         als_tilt(sm, a, side, nullptr);
       // every CTA of a cluster is done with its copy of the last reduced
       // metric before any writes the next one, and all blocks are in before

@@ -198,7 +198,7 @@ static __device__ void als_matvec(AlsShared& sm, const double2* A, const float4*
 static __device__ void low_normalise(AlsShared& sm, double2* v, int n) {
   double s = 0.0;
   for (int i = threadIdx.x; i < n; i += NTU_CTA) s += cabs2(v[i]);
-  s = block_sum(s, sm.red);
+  s = block_sum<true>(s, sm.red);
   const double f = s > 0.0 ? rsqrt(s) : 0.0;
   for (int i = threadIdx.x; i < n; i += NTU_CTA) v[i] = cscale(v[i], f);
   __syncthreads();
@@ -238,8 +238,8 @@ static __device__ __noinline__ int als_solve_certified(AlsShared& sm, const AlsA
   double fs = 0.0, low = 0.0;
   for (int idx = tid; idx < n * n; idx += NTU_CTA) fs += cabs2(gX[idx]);
   for (int i = tid; i < n; i += NTU_CTA) low = fmax(low, gX[(size_t)i * n + i].x);
-  fs = sqrt(block_sum(fs, sm.red)) * (1.0 + 1e-12);
-  low = block_max(low, sm.red);
+  fs = sqrt(block_sum<true>(fs, sm.red)) * (1.0 + 1e-12);
+  low = block_max<true>(low, sm.red);
   double B = fs < bmax ? fs : bmax;
   if (!(B > 0x1p-900) || !(B < 0x1p900)) return 0;
   const int e = ilogb(B);
@@ -257,7 +257,7 @@ static __device__ __noinline__ int als_solve_certified(AlsShared& sm, const AlsA
         s += cmulc(sm.p[i], sm.ap[i]).x;
         sm.p[i] = sm.ap[i];
       }
-      low = fmax(low, block_sum(s, sm.red));
+      low = fmax(low, block_sum<true>(s, sm.red));
     }
     for (int t = 0; t < 2; ++t) {
       const double b = (t ? 1.08 : 1.01) * low;
@@ -282,7 +282,7 @@ static __device__ __noinline__ int als_solve_certified(AlsShared& sm, const AlsA
       sm.p[i] = sm.y[i];
       f0 += cmulc(sm.y[i], jv[i]).x;
     }
-    f0 = block_sum(f0, sm.red);
+    f0 = block_sum<true>(f0, sm.red);
     // u_q = (thr / gX)^q x and F_2q = thr u_q^H u_{q-1}, with thr at k = kmin + 1;
     // a larger k rescales F_p by 10^-p per step (F in units of that thr)
     const double thr1 = als_tau(kmin) * low * (1.0 - 1e-9);
@@ -302,8 +302,8 @@ static __device__ __noinline__ int als_solve_certified(AlsShared& sm, const AlsA
           s += cmulc(u, sm.y2[i]).x;
           uu += cabs2(u);
         }
-        F[q] = thr1 * block_sum(s, sm.red);
-        uu = block_sum(uu, sm.red);
+        F[q] = thr1 * block_sum<true>(s, sm.red);
+        uu = block_sum<true>(uu, sm.red);
         rp = rho;
         rho = F[q] / uu;                                    // >= lambda_min
         if (!(F[q] > 0.0) || !isfinite(uu)) return 0;
@@ -680,10 +680,10 @@ static __device__ void tri_orthonormalise(AlsShared& sm, double* W, int n, int m
         __syncthreads();
       }
       double mx = tid < n ? fabs(wj[tid]) : 0.0;
-      mx = block_max(mx, sm.red);
+      mx = block_max<true>(mx, sm.red);
       const double f = mx > 0.0 && isfinite(mx) ? 1.0 / mx : 0.0;
       const double x = tid < n ? wj[tid] * f : 0.0;
-      const double s = block_sum(x * x, sm.red);
+      const double s = block_sum<true>(x * x, sm.red);
       if (tid < n) wj[tid] = s > 0.0 ? x * rsqrt(s) : 0.0;
       __syncthreads();
     }
@@ -794,7 +794,7 @@ static __device__ __noinline__ void als_solve_spectrum(AlsShared& sm, const AlsA
     sm.p[i] = r > 0.0 ? make_double2(z.x / r, z.y / r) : make_double2(1.0, 0.0);
     mxe = fmax(mxe, fmax(fabs(dv[i]), r));
   }
-  mxe = block_max(mxe, sm.red);
+  mxe = block_max<true>(mxe, sm.red);
   const bool finite = isfinite(mxe) && mxe > 0.0;
   int se = finite ? ilogb(mxe) : 0;
   se = se < -1000 ? -1000 : (se > 1000 ? 1000 : se);

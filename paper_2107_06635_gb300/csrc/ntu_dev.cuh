@@ -204,6 +204,13 @@ __device__ __forceinline__ double warp_max(double v) {
 }
 
 // Sum over the CTA; every thread gets the result.  sbuf: >= NTU_WARPS*2 doubles.
+// LONE: thread 0 adds the warps' sums (in their order, so the same bits) where
+// otherwise every warp does.  Eight FP64 adds in eight warps take longer than in
+// one and a barrier more where a CTA has the SM to itself (the FP64 contexts:
+// 6.6 against 6.0 ms for a cell step at D = 3, with the tilts' roots in one warp),
+// not where three CTAs fill each other's waits (43.0 against 43.4 ms for 912
+// updates at D = 8).
+template <bool LONE = false>
 __device__ __forceinline__ double block_sum(double v, double* sbuf) {
   v = warp_sum(v);
   int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -211,9 +218,14 @@ __device__ __forceinline__ double block_sum(double v, double* sbuf) {
   if (l == 0) sbuf[w] = v;
   __syncthreads();
   double t = 0.0;
+  if (!LONE || threadIdx.x == 0) {
 #pragma unroll
-  for (int i = 0; i < NTU_WARPS; ++i) t += sbuf[i];
-  return t;
+    for (int i = 0; i < NTU_WARPS; ++i) t += sbuf[i];
+  }
+  if (!LONE) return t;
+  if (threadIdx.x == 0) sbuf[0] = t;
+  __syncthreads();
+  return sbuf[0];
 }
 __device__ __forceinline__ double2 block_sum2(double2 v, double* sbuf) {
   v = warp_sum2(v);
@@ -226,6 +238,7 @@ __device__ __forceinline__ double2 block_sum2(double2 v, double* sbuf) {
   for (int i = 0; i < NTU_WARPS; ++i) { t.x += sbuf[2 * i]; t.y += sbuf[2 * i + 1]; }
   return t;
 }
+template <bool LONE = false>
 __device__ __forceinline__ double block_min(double v, double* sbuf) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = fmin(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -234,10 +247,16 @@ __device__ __forceinline__ double block_min(double v, double* sbuf) {
   if (l == 0) sbuf[w] = v;
   __syncthreads();
   double t = sbuf[0];
+  if (!LONE || threadIdx.x == 0) {
 #pragma unroll
-  for (int i = 1; i < NTU_WARPS; ++i) t = fmin(t, sbuf[i]);
-  return t;
+    for (int i = 1; i < NTU_WARPS; ++i) t = fmin(t, sbuf[i]);
+  }
+  if (!LONE) return t;
+  if (threadIdx.x == 0) sbuf[NTU_WARPS] = t;
+  __syncthreads();
+  return sbuf[NTU_WARPS];
 }
+template <bool LONE = false>
 __device__ __forceinline__ double block_max(double v, double* sbuf) {
   v = warp_max(v);
   int w = threadIdx.x >> 5, l = threadIdx.x & 31;
@@ -245,9 +264,14 @@ __device__ __forceinline__ double block_max(double v, double* sbuf) {
   if (l == 0) sbuf[w] = v;
   __syncthreads();
   double t = sbuf[0];
+  if (!LONE || threadIdx.x == 0) {
 #pragma unroll
-  for (int i = 1; i < NTU_WARPS; ++i) t = fmax(t, sbuf[i]);
-  return t;
+    for (int i = 1; i < NTU_WARPS; ++i) t = fmax(t, sbuf[i]);
+  }
+  if (!LONE) return t;
+  if (threadIdx.x == 0) sbuf[NTU_WARPS] = t;
+  __syncthreads();
+  return sbuf[NTU_WARPS];
 }
 
 // Error codes a kernel may raise through the status word (same values as
@@ -461,12 +485,20 @@ __device__ inline void cta_svd_cols(SvdSmem& S, int m, int n, int phase) {
             double2 ap = S.A[p * 32 + r], aq = S.A[q * 32 + r];
             al += cabs2(ap); be += cabs2(aq); ga = cfmac(ap, aq, ga);
           }
-#pragma unroll
-          for (int o = 8; o > 0; o >>= 1) {
-            al += __shfl_xor_sync(mask, al, o);
-            be += __shfl_xor_sync(mask, be, o);
-            ga.x += __shfl_xor_sync(mask, ga.x, o);
-            ga.y += __shfl_xor_sync(mask, ga.y, o);
+          // the four sums over the 16 lanes together (5 FP64 adds instead of
+          // 16, the same pairings): a quarter of the lanes ends with each
+          {
+            const bool h8 = (lane & 8) != 0, h4 = (lane & 4) != 0;
+            const double v0 = (h8 ? ga.x : al) + __shfl_xor_sync(mask, h8 ? al : ga.x, 8);
+            const double v1 = (h8 ? ga.y : be) + __shfl_xor_sync(mask, h8 ? be : ga.y, 8);
+            double t = (h4 ? v1 : v0) + __shfl_xor_sync(mask, h4 ? v0 : v1, 4);
+            t += __shfl_xor_sync(mask, t, 2);
+            t += __shfl_xor_sync(mask, t, 1);
+            const int b = tid & 16;
+            al = __shfl_sync(mask, t, b);
+            be = __shfl_sync(mask, t, b + 4);
+            ga.x = __shfl_sync(mask, t, b + 8);
+            ga.y = __shfl_sync(mask, t, b + 12);
           }
           const double g2 = cabs2(ga);
           const double rg = g2 > 0.0 ? rsqrt(g2) : 0.0;      // 1 / |<a_p, a_q>|
