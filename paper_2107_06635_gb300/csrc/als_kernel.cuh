@@ -1070,7 +1070,7 @@ static __device__ void als_mirror(double2* gX, int nA) {
 // larger tau.  The result is written to sm.MA (side 0) or sm.MB (side 1).
 // The arithmetic of the implicit QR (tridiag_qr) and of its rotations is kept
 // to the last bit, as for the shifted-Cholesky solves (als_slow.cuh); one thread
-// took 8 to 11 ms a solve at n = 64 to 72 with all of it in one chain.  Now warp
+// took 11.6 ms a solve at n = 72 with all of it in one chain (7.7 now).  Now warp
 // 0 runs the sweeps on T in shared memory (both quotients of a rotation in one
 // division, the deflation test a lane per entry) while warp 1 applies the sweep
 // before to y, its real and imaginary parts in two lanes; the selection takes a

