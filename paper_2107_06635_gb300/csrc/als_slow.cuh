@@ -820,6 +820,8 @@ static __device__ __noinline__ void als_solve_spectrum(AlsShared& sm, const AlsA
   __syncthreads();
   const int kmin = a.kmin < 0 ? 0 : a.kmin, kmax = a.kmax > 20 ? 20 : a.kmax, nk = kmax - kmin + 1;
   int* cnt = reinterpret_cast<int*>(sm.ph);                 // eigenvalues below tau_k lambda_max
+  int* ndrop = cnt + 32;                                    // pairs dropped (a word of its own: every
+                                                            // warp still reads sm.flag then)
   double* lim = reinterpret_cast<double*>(sm.ph + 16);      // [lower bound, lambda_max]
   if (wid == 0) {
     double lo = INFINITY, hi = -INFINITY;
@@ -934,10 +936,10 @@ static __device__ __noinline__ void als_solve_spectrum(AlsShared& sm, const AlsA
         if (sm.eps0 - (all - part) <= sm.eps0 - all + 1e-14 * sm.eps0) break;
       }
       sm.tau_sel = als_tau(kmin + k);
-      sm.flag = cnt[k];
+      *ndrop = cnt[k];
     }
     __syncthreads();
-    const int drop = sm.flag;
+    const int drop = *ndrop;
     if (m == n) {
       double2 v = cz();
       if (tid < n)
