@@ -65,23 +65,30 @@ __device__ __forceinline__ bool low_pair(int m, int q, int pos, int& i, int& k) 
 }
 
 // Whether sg (gX - shift I), sg = 1 or -1, is positive definite: an L D L^H
-// factorisation in double-FP32 arithmetic (2^-46 relative, covered
-// by the 1e-12 lambda_max that the caller allows for in the shift) succeeds.  A warp's
-// double-FP32 complex multiply-add takes 48 issue slots where the FP64 one
+// factorisation of it minus a margin I in double-FP32 arithmetic succeeds.  Every
+// entry is renormalised after each update (|lo| <= 2^-24 |hi|: a pivot that has
+// cancelled to the size of its low part would otherwise be tested by a high
+// part without meaning), so an update of a_ik errs by at most 2^-46 of
+// 5 |c_i c_k| / d + sqrt(a_ii a_kk), and n of them perturb a positive definite
+// matrix by a matrix of norm below 4 (n + 2) 2^-46 tr.  That is the margin, with
+// the trace bounded by tr gX (sg = 1) or n shift (sg = -1): success proves
+// it, and a matrix that is definite by less goes to the spectrum.  A warp's
+// double-FP32 complex multiply-add takes 60 issue slots where the FP64 one
 // holds its pipe for 256 cycles; one barrier per step, the reciprocal pivot
 // from FP32 and one double-FP32 correction by every thread.
 template <bool SH>
 static __device__ int low_certify(AlsShared& sm, int n, const double2* gX, void* buf, double shift,
-                                  int e, double sg) {
+                                  double tr, int e, double sg) {
   const int tid = threadIdx.x;
   float4* A = reinterpret_cast<float4*>(buf);
   const LowTri<SH> L = {nullptr, n};
   const double f = sg * pow2i(-e);                          // entries of about 1 at most
+  const double sh = shift + sg * 4.0 * (n + 2) * 0x1p-46 * (sg > 0.0 ? tr : n * shift);
   for (int idx = tid; idx < n * n; idx += NTU_CTA) {
     const int i = idx % n, k = idx / n;
     if (i < k) continue;
     double2 v = gX[idx];
-    if (i == k) v = make_double2(v.x - shift, 0.0);
+    if (i == k) v = make_double2(v.x - sh, 0.0);
     A[L.off(k) + i] = df_split(cscale(v, f));
   }
   __syncthreads();
@@ -112,6 +119,8 @@ static __device__ int low_certify(AlsShared& sm, int n, const double2* gX, void*
         float4* x = A + L.off(j + 1 + k) + j + 1 + i;
         float4 acc = *x;
         df_cmac<true>(acc, c[j + 1 + k], i == q ? v1 : v2); // a -= (c_i / d) conj(c_k)
+        df_renorm(acc.x, acc.z);
+        df_renorm(acc.y, acc.w);
         *x = acc;
       }
     }
@@ -235,15 +244,19 @@ static __device__ __noinline__ int als_solve_certified(AlsShared& sm, const AlsA
   const LowTri<SH> L = {SH ? sm.S.A : gC, n};
   void* buf = SH ? (void*)sm.S.A : (void*)gC;
   const int kmin = a.kmin < 0 ? 0 : a.kmin, kmax = a.kmax > 20 ? 20 : a.kmax;
-  double fs = 0.0, low = 0.0;
+  double fs = 0.0, low = 0.0, tr = 0.0;
   for (int idx = tid; idx < n * n; idx += NTU_CTA) fs += cabs2(gX[idx]);
-  for (int i = tid; i < n; i += NTU_CTA) low = fmax(low, gX[(size_t)i * n + i].x);
+  for (int i = tid; i < n; i += NTU_CTA) {
+    low = fmax(low, gX[(size_t)i * n + i].x);
+    tr += gX[(size_t)i * n + i].x;
+  }
   fs = sqrt(block_sum<true>(fs, sm.red)) * (1.0 + 1e-12);
   low = block_max<true>(low, sm.red);
+  tr = block_sum<true>(tr, sm.red);
   double B = fs < bmax ? fs : bmax;
   if (!(B > 0x1p-900) || !(B < 0x1p900)) return 0;
   const int e = ilogb(B);
-  const int all = low_certify<SH>(sm, n, gX, buf, (als_tau(kmin) + 1e-12) * B, e, 1.0);
+  const int all = low_certify<SH>(sm, n, gX, buf, (als_tau(kmin) + 1e-12) * B, tr, e, 1.0);
   if (!all) {
     // lambda_max from below by eight steps of the power iteration on J, and
     // from above, where it holds, by 1.01 times that
@@ -261,7 +274,7 @@ static __device__ __noinline__ int als_solve_certified(AlsShared& sm, const AlsA
     }
     for (int t = 0; t < 2; ++t) {
       const double b = (t ? 1.08 : 1.01) * low;
-      if (b < B && low_certify<SH>(sm, n, gX, buf, b * (1.0 - 1e-12), e, -1.0)) { B = b; break; }
+      if (b < B && low_certify<SH>(sm, n, gX, buf, b, tr, e, -1.0)) { B = b; break; }
       __syncthreads();
     }
   }
@@ -337,7 +350,7 @@ static __device__ __noinline__ int als_solve_certified(AlsShared& sm, const AlsA
     }
     if (!done) return 0;
     __syncthreads();
-    if (!low_certify<SH>(sm, n, gX, buf, sig, e, 1.0)) return 0;
+    if (!low_certify<SH>(sm, n, gX, buf, sig, tr, e, 1.0)) return 0;
   }
   double2* M = side == 0 ? sm.MA : sm.MB;
   for (int i = tid; i < n; i += NTU_CTA) M[i] = sm.y[i];

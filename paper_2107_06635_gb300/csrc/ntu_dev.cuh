@@ -367,6 +367,13 @@ __device__ __forceinline__ void df_mac1(float& sh, float& sl, float xh, float xl
   sh = t;
   sl = __fadd_rn(sl, __fadd_rn(err, e));
 }
+// (h, l) with the same sum and |l| <= 2^-24 |h|, whichever was the larger
+__device__ __forceinline__ void df_renorm(float& h, float& l) {
+  const float t = __fadd_rn(h, l);
+  const float z = __fsub_rn(t, h);
+  l = __fadd_rn(__fsub_rn(h, __fsub_rn(t, z)), __fsub_rn(l, z));
+  h = t;
+}
 // acc += a * b, or conj(a) * b with CONJ
 template <bool CONJ>
 __device__ __forceinline__ void df_cmac(float4& acc, float4 a, float4 b) {

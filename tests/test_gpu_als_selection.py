@@ -60,3 +60,18 @@ def test_nothing_dropped_through_the_spectrum(D, kmax):
     lam = np.concatenate([np.geomspace(1.003 * 10.0 ** -kmax, 0.3, n - 1), [1.0]])
     paths = _check(D, lam, 48, 4, kmax, 5 * D + kmax, 3e-9)
     assert paths["als_eigen"] == 2 * 48
+
+
+@pytest.mark.parametrize("D", [2, 4, 7, 8])
+@pytest.mark.parametrize("k", [7, 8, 9, 10])
+@pytest.mark.parametrize("fac", [0.3, 3.0])
+@pytest.mark.parametrize("kmin", [4, None])
+def test_isolated_eigenvalue_next_to_a_tolerance(D, k, fac, kmin):
+    """One eigenvalue at fac 10^-k lambda_max, the others above 10^-2: the
+    largest tolerance that keeps it is 10^-k or 10^-(k+1), and a certificate at
+    10^-k is right only for fac > 1.  kmin None: 10^-k is the first candidate.
+    Dropping the pair costs at least 3e-11 / n_A of eps0, far above 1e-14.  Two
+    solves a side of condition 1 / lambda_min, each good to n_A 2^-53 times it."""
+    n = D * D
+    lam = np.concatenate([[fac * 10.0 ** -k], np.geomspace(1e-2, 1.0, n - 1)])
+    _check(D, lam, 20, k if kmin is None else kmin, k + 2, 1000 * k + D, 4.0 * n * 2.0 ** -53 / lam[0])
