@@ -655,21 +655,22 @@ static cudaError_t env_chain_oz64(ntu_ctx* c, int n, const double2* Ta, const do
     const int m = n - i0 < P.oz64.items ? n - i0 : P.oz64.items;
     const double2 *ta = Ta + i0 * P.szT, *tb = Tb + i0 * P.szT;
     const double2 *qa = QA + i0 * P.szQ, *qb = QB + i0 * P.szQ;
+    RG(oz64_begin(c));
     RG(run_gram<double2>(c, P.eL, m, tb, EL));
     RG(run_gram<double2>(c, P.eR, m, ta, ER));
-    RG(launch_oz64(c, P.eTL, 0, m, tb, tb, (double2*)W.ETL));
-    RG(launch_oz64(c, P.eBL, 0, m, tb, tb, (double2*)W.EBL));
-    RG(launch_oz64(c, P.eTR, 0, m, ta, ta, (double2*)W.ETR));
-    RG(launch_oz64(c, P.eBR, 0, m, ta, ta, (double2*)W.EBR));
+    RG(launch_oz64(c, P.eTL, 0, -1, m, tb, tb, (double2*)W.ETL));
+    RG(launch_oz64(c, P.eBL, 0, -1, m, tb, tb, (double2*)W.EBL));
+    RG(launch_oz64(c, P.eTR, 0, -1, m, ta, ta, (double2*)W.ETR));
+    RG(launch_oz64(c, P.eBR, 0, -1, m, ta, ta, (double2*)W.EBR));
     RG(run_gemm<double2>(c, P.y, m, qa, EL, Y));
-    RG(launch_oz64(c, P.t1, 1, m, Y, qa, T1));
-    RG(launch_oz64(c, P.t2, 2, m, (double2*)W.ETL, T1, T2));
-    RG(launch_oz64(c, P.h, 2, m, (double2*)W.EBL, T2, HL));
+    RG(launch_oz64(c, P.t1, 1, 0, m, Y, qa, T1));
+    RG(launch_oz64(c, P.t2, 2, 1, m, (double2*)W.ETL, T1, T2));
+    RG(launch_oz64(c, P.h, 2, 2, m, (double2*)W.EBL, T2, HL));
     RG(run_gemm<double2>(c, P.y, m, qb, ER, Y));
-    RG(launch_oz64(c, P.t1, 1, m, Y, qb, T1));
-    RG(launch_oz64(c, P.t2, 2, m, (double2*)W.ETR, T1, T2));
-    RG(launch_oz64(c, P.h, 2, m, (double2*)W.EBR, T2, HR));
-    RG(launch_oz64(c, P.join, 3, m, HL, HR, graw + i0 * P.szG));
+    RG(launch_oz64(c, P.t1, 1, 3, m, Y, qb, T1));
+    RG(launch_oz64(c, P.t2, 2, 4, m, (double2*)W.ETR, T1, T2));
+    RG(launch_oz64(c, P.h, 2, 5, m, (double2*)W.EBR, T2, HR));
+    RG(launch_oz64(c, P.join, 3, 6, m, HL, HR, graw + i0 * P.szG));
   }
   return cudaSuccess;
 }

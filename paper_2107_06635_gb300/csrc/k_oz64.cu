@@ -17,7 +17,15 @@
 // of 12 to 32 terms were up to 1.7 times less accurate than the FP64 chain).
 // The epilogue joins the levels as integers and rounds once to FP64, without
 // FP64 instructions (one holds the pipe of a quarter of the SM for 64 cycles).
-// What is left is the operands' rounding to 2^-55 of their row's largest entry:
+// What is left is the operands' rounding to 2^-55 of their row's largest entry.
+// A floating-point sum does not care how its index is scaled (a bond whose leg
+// grows on one site as its partner falls on the other), a rounding relative to
+// a row does, so the terms are balanced first: with a_k and b_k the exponents of
+// the largest entries of term k on either side, the left operand is taken times
+// 2^((b_k - a_k) / 2) and the right one divided by it, in the exponents alone.
+// (Scales 1 .. 1e-8 on a leg and their inverses on its partner cost the metric
+// all its digits without.)  The edges are Gram products: a_k = b_k.
+// With that,
 // relative to 113-bit sums the metric at D = 2 to 4 is off by 1e-16 to 1e-15
 // where the FP64 chain was off by 3e-16 to 2.3e-15.
 //
@@ -63,6 +71,7 @@ constexpr int ZEPI = 16, ZTHREADS = 64 + 32 * ZEPI;
 constexpr size_t ZSMEM = (size_t)ZSTAGES * ZSTAGE + 1024 + 256;
 constexpr long long ZWAIT = 1ll << 28;
 constexpr int ZNAN = 20000;                           // exponent of a row with a non-finite entry
+constexpr int ZNONE = -(1 << 24), ZINF = 1 << 24;     // exponent of 0, of a non-finite entry
 static_assert(ZSMEM <= 227 * 1024, "shared memory budget");
 
 // K-major tile whose rows are 64 bytes, written by TMA with the 64-byte
@@ -314,25 +323,75 @@ struct Oz64Slice {
   __nv_bfloat16* out;                    // [item][7][rowsP][2 Kh]
   int* ex;                               // [item][epitch] row exponents
   int epitch;
-  unsigned* mx;                          // [item][epitch] high words of the largest entries
+  int* mx;                               // [item][epitch] exponents of the largest entries
+  int* cm;                               // [item][2][kpitch] exponents of the terms, left and
+  int kpitch;                            // right (NULL: not balanced)
 };
 
-// Largest |Re|, |Im| of every row (the high word of its bits), for rows of
-// more than 64 terms; 32 rows x 8 terms per pass, coalesced along the rows.
+// Biased exponent of the leading bit of the larger part of v (below 1 for
+// subnormals).
+__device__ __forceinline__ int oz64_exp(double2 v) {
+  const unsigned h = max((unsigned)__double2hiint(v.x) & 0x7fffffffu, (unsigned)__double2hiint(v.y) & 0x7fffffffu);
+  const int e = (int)(h >> 20);
+  if (e == 0) {
+    const long long m = 0xfffffffffffffll;
+    const long long b = max(__double_as_longlong(v.x) & m, __double_as_longlong(v.y) & m);
+    return b ? 12 - __clzll(b) : ZNONE;
+  }
+  return e == 0x7ff ? ZINF : e;
+}
+
+// Exponent of the factor of term k: (b_k - a_k) / 2 on the left operand, its
+// negative on the right one; 0 where a side has no finite non-zero entry.
+__device__ __forceinline__ int oz64_factor(const Oz64Slice& s, long long z, int k) {
+  if (!s.cm || k >= s.K) return 0;
+  const int* c = s.cm + z * 2 * s.kpitch + k;
+  const int a = c[0], b = c[s.kpitch];
+  if (a < -4096 || b < -4096 || a > 4096 || b > 4096) return 0;
+  const int f = (b - a) >> 1;
+  return s.doubled ? f : -f;
+}
+
+// Exponents of the largest entries of every term of both operands: a warp
+// takes eight terms of 128 rows, coalesced along the rows.
+__global__ void __launch_bounds__(256) k_oz64_terms(Oz64Slice left, Oz64Slice right, int lblocks) {
+  const bool lt = (int)blockIdx.x < lblocks;
+  const Oz64Slice& s = lt ? left : right;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int r0 = ((int)blockIdx.x - (lt ? 0 : lblocks)) * 128 + lane, k0 = blockIdx.y * 64 + w;
+  const double2* p = s.src + (long long)blockIdx.z * s.s_src;
+  int* c = s.cm + ((long long)blockIdx.z * 2 + (lt ? 0 : 1)) * s.kpitch;
+  int off[4];
+#pragma unroll
+  for (int t = 0; t < 4; ++t) off[t] = r0 + 32 * t < s.rows ? s.row[r0 + 32 * t] : -1;
+#pragma unroll 2
+  for (int i = 0; i < 8; ++i) {
+    const int k = k0 + 8 * i;
+    if (k >= s.K) break;
+    const int kk = s.kk[k];
+    int e = ZNONE;
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+      if (off[t] >= 0) e = max(e, oz64_exp(p[off[t] + kk]));
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) atomicMax(c + k, e);
+  }
+}
+
+// Exponent of the largest entry of every row, for rows of more than 64 terms;
+// 32 rows x 8 terms per pass, coalesced along the rows.
 __global__ void __launch_bounds__(256) k_oz64_max(Oz64Slice s) {
-  __shared__ unsigned red[8][32];
+  __shared__ int red[8][32], fac[256];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int r = blockIdx.x * 32 + lane, k0 = blockIdx.y * 256;
-  unsigned m = 0;
+  fac[threadIdx.x] = oz64_factor(s, blockIdx.z, k0 + (int)threadIdx.x);
+  __syncthreads();
+  int m = ZNONE;
   if (r < s.rows) {
     const double2* p = s.src + (long long)blockIdx.z * s.s_src + s.row[r];
     const int k1 = k0 + 256 < s.K ? k0 + 256 : s.K;
 #pragma unroll 4
-    for (int k = k0 + w; k < k1; k += 8) {
-      const double2 v = p[s.kk[k]];
-      m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu,
-                     (unsigned)__double2hiint(v.y) & 0x7fffffffu));
-    }
+    for (int k = k0 + w; k < k1; k += 8) m = max(m, oz64_exp(p[s.kk[k]]) + fac[k - k0]);
   }
   red[w][lane] = m;
   __syncthreads();
@@ -342,17 +401,17 @@ __global__ void __launch_bounds__(256) k_oz64_max(Oz64Slice s) {
   }
 }
 
-// x 2^(54 - e) rounded to the nearest integer, e = em - 1022 (em the biased
-// exponent of the row's largest entry), from the bits.
-__device__ __forceinline__ long long oz64_fix(double x, int em) {
+// x 2^(f + 54 - e) rounded to the nearest integer, e = em - 1022 (em the biased
+// exponent of the row's largest entry times its factor), from the bits.
+__device__ __forceinline__ long long oz64_fix(double x, int em, int f) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   int ex = (int)(b >> 52) & 0x7ff;
   unsigned long long m = b & 0xfffffffffffffull;
   if (ex) m |= 0x10000000000000ull;
   else ex = 1;
-  const int sh = em - 1 - ex;                             // >= -1
-  long long v = sh < 0 ? (long long)(m << 1)
-                       : (sh == 0 ? (long long)m : (sh < 56 ? (long long)((m + (1ull << (sh - 1))) >> sh) : 0ll));
+  const int sh = em - 1 - (ex + f);                       // >= -1, below for subnormals
+  const long long v = sh <= 0 ? (long long)(m << (-sh & 63))
+                              : (sh < 56 ? (long long)((m + (1ull << (sh - 1))) >> sh) : 0ll);
   return (long long)b < 0 ? -v : v;
 }
 
@@ -360,14 +419,15 @@ __device__ __forceinline__ long long oz64_fix(double x, int em) {
 // written as 16-byte runs of eight terms of every slice.
 __global__ void __launch_bounds__(256) k_oz64_slice(Oz64Slice s) {
   __shared__ double2 tile[64 * 33];
-  __shared__ unsigned red[8][32];
-  __shared__ int em[32];
+  __shared__ int red[8][32], em[32], fac[64];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int r0 = blockIdx.x * 32, k0 = blockIdx.y * 64;
   const long long z = blockIdx.z;
   {
     const int r = r0 + lane;
-    unsigned m = 0;
+    int m = ZNONE;
+    if (threadIdx.x < 64) fac[threadIdx.x] = oz64_factor(s, z, k0 + (int)threadIdx.x);
+    __syncthreads();
     const double2* p = s.src + z * s.s_src + (r < s.rows ? s.row[r] : 0);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -376,21 +436,19 @@ __global__ void __launch_bounds__(256) k_oz64_slice(Oz64Slice s) {
       if (r < s.rows && k0 + k < s.K) v = p[s.kk[k0 + k]];
       if (s.conj) v.y = -v.y;
       tile[k * 33 + lane] = v;
-      m = max(m, max((unsigned)__double2hiint(v.x) & 0x7fffffffu,
-                     (unsigned)__double2hiint(v.y) & 0x7fffffffu));
+      m = max(m, oz64_exp(v) + fac[k]);
     }
     red[w][lane] = m;
     __syncthreads();
     if (w == 0) {
       if (s.mx) {
-        m = r < s.rows ? s.mx[z * s.epitch + r] : 0;
+        m = r < s.rows ? s.mx[z * s.epitch + r] : ZNONE;
       } else {
         for (int i = 1; i < 8; ++i) m = max(m, red[i][lane]);
       }
-      const int e = max((int)(m >> 20), 1);
+      const int e = m < -8192 ? 1 : m;                      // a row of zeros
       em[lane] = e;
-      if (blockIdx.y == 0 && r < s.epitch)
-        s.ex[z * s.epitch + r] = e >= 0x7ff ? ZNAN : e - 1022;
+      if (blockIdx.y == 0 && r < s.epitch) s.ex[z * s.epitch + r] = e > 8192 ? ZNAN : e - 1022;
     }
     __syncthreads();
   }
@@ -409,7 +467,7 @@ __global__ void __launch_bounds__(256) k_oz64_slice(Oz64Slice s) {
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         const double2 v = tile[(kg + 2 * p + u) * 33 + rl];
-        long long x = e >= 0x7ff ? 0 : oz64_fix(c ? v.y : v.x, e);
+        long long x = e > 8192 ? 0 : oz64_fix(c ? v.y : v.x, e, fac[kg + 2 * p + u]);
 #pragma unroll
         for (int i = ZS - 1; i >= 0; --i) {
           const int d = i ? (int)((unsigned)(x + 128) & 255u) - 128 : (int)x;
@@ -497,6 +555,8 @@ void oz64_init(ntu_ctx* c) {
     ra = g.rowsA / 2 > ra ? g.rowsA / 2 : ra;
     rb = g.rowsB > rb ? g.rowsB : rb;
   }
+  z.kpitch = 1;
+  for (const GemmOp* o : ops) z.kpitch = o->Kd > z.kpitch ? o->Kd : z.kpitch;
   a = (a + 1023) / 1024 * 1024;
   b = (b + 1023) / 1024 * 1024;
   // items at a time: enough to fill the SMs, within about 2 GB.  Rows beyond
@@ -505,7 +565,8 @@ void oz64_init(ntu_ctx* c) {
   long long items = (2ll << 30) / (a + b);
   if (items < 1) items = 1;
   if (items > c->cfg.max_batch) items = c->cfg.max_batch;
-  const long long ebytes = items * (ra + 2LL * rb + ra) * 4;
+  const long long tbytes = items * OZ64_BALANCED * 2LL * z.kpitch * 4;
+  const long long ebytes = items * (ra + 2LL * rb + ra) * 4 + tbytes;
   void* base = nullptr;
   if (cudaMalloc(&base, items * (a + b) + ebytes) != cudaSuccess) {
     cudaGetLastError();                                    // no room: the SIMT path
@@ -516,7 +577,8 @@ void oz64_init(ntu_ctx* c) {
   z.SB = z.SA + items * a;
   z.eA = (int*)(z.SB + items * b);
   z.eB = z.eA + items * ra;
-  z.mx = (unsigned*)(z.eB + items * rb);
+  z.cm = z.eB + items * rb;
+  z.mx = z.cm + tbytes / 4;
   int st = NTU_OK;
   for (int i = 0; i < 4 && st == NTU_OK; ++i) {
     Oz64Geo& g = z.geo[i];
@@ -531,9 +593,15 @@ void oz64_free(ntu_ctx* c) {
   c->plan.oz64.base = nullptr;
 }
 
-static cudaError_t oz64_slice(ntu_ctx* c, const GemmOp& op, const Oz64Geo& g, int n, bool left,
+// Empties the term exponents of a pass's balanced products.
+cudaError_t oz64_begin(ntu_ctx* c) {
+  const Oz64& z = c->plan.oz64;
+  return cudaMemsetAsync(z.cm, 0x80, sizeof(int) * (size_t)z.items * OZ64_BALANCED * 2 * z.kpitch, c->stream);
+}
+
+static Oz64Slice oz64_operand(ntu_ctx* c, const GemmOp& op, const Oz64Geo& g, int slot, bool left,
                               const double2* src) {
-  Oz64& z = c->plan.oz64;
+  const Oz64& z = c->plan.oz64;
   const int* t = c->plan.d_tab;
   Oz64Slice s;
   s.src = src;
@@ -549,11 +617,16 @@ static cudaError_t oz64_slice(ntu_ctx* c, const GemmOp& op, const Oz64Geo& g, in
   s.out = reinterpret_cast<__nv_bfloat16*>(left ? z.SA : z.SB);
   s.ex = left ? z.eA : z.eB;
   s.epitch = left ? g.rowsA / 2 : g.rowsB;
-  s.mx = nullptr;
+  s.mx = g.Kh > 64 ? z.mx : nullptr;
+  s.cm = slot < 0 ? nullptr : z.cm + (size_t)slot * z.items * 2 * z.kpitch;
+  s.kpitch = z.kpitch;
+  return s;
+}
+
+static cudaError_t oz64_slice(ntu_ctx* c, const Oz64Slice& s, int n) {
   const unsigned bx = (unsigned)((s.rows + 31) / 32);
-  if (s.Kh > 64) {
-    s.mx = z.mx;
-    cudaError_t e = cudaMemsetAsync(z.mx, 0, sizeof(unsigned) * (size_t)n * s.epitch, c->stream);
+  if (s.mx) {
+    cudaError_t e = cudaMemsetAsync(s.mx, 0x80, sizeof(int) * (size_t)n * s.epitch, c->stream);
     if (e != cudaSuccess) return e;
     k_oz64_max<<<dim3(bx, (unsigned)((s.K + 255) / 256), (unsigned)n), 256, 0, c->stream>>>(s);
     e = after_launch(c, "k_oz64_max");
@@ -563,13 +636,23 @@ static cudaError_t oz64_slice(ntu_ctx* c, const GemmOp& op, const Oz64Geo& g, in
   return after_launch(c, "k_oz64_slice");
 }
 
-// C = A B of one plan GEMM for n <= oz64.items items (geometry index gi).
-cudaError_t launch_oz64(ntu_ctx* c, const GemmOp& op, int gi, int n, const double2* A,
+// C = A B of one plan GEMM for n <= oz64.items items (geometry index gi; slot:
+// that of its term exponents among the pass's balanced products, -1 for a Gram
+// product).
+cudaError_t launch_oz64(ntu_ctx* c, const GemmOp& op, int gi, int slot, int n, const double2* A,
                         const double2* B, double2* C) {
   Oz64& z = c->plan.oz64;
   const Oz64Geo& g = z.geo[gi];
-  cudaError_t e = oz64_slice(c, op, g, n, true, A);
-  if (e == cudaSuccess) e = oz64_slice(c, op, g, n, false, B);
+  const Oz64Slice sa = oz64_operand(c, op, g, slot, true, A), sb = oz64_operand(c, op, g, slot, false, B);
+  cudaError_t e = cudaSuccess;
+  if (slot >= 0) {
+    const int la = (sa.rows + 127) / 128, lb = (sb.rows + 127) / 128;
+    k_oz64_terms<<<dim3((unsigned)(la + lb), (unsigned)((op.Kd + 63) / 64), (unsigned)n), 256, 0, c->stream>>>(
+        sa, sb, la);
+    e = after_launch(c, "k_oz64_terms");
+  }
+  if (e == cudaSuccess) e = oz64_slice(c, sa, n);
+  if (e == cudaSuccess) e = oz64_slice(c, sb, n);
   if (e != cudaSuccess) return e;
   Oz64Args a;
   const int* t = c->plan.d_tab;

@@ -57,6 +57,7 @@ struct TcOp {
 // one plan GEMM (rowsA real rows of the doubled left operand, rowsB rows of the
 // right one, Kh padded complex terms) and the scratch shared by all of them.
 constexpr int OZ64_SLICES = 7;
+constexpr int OZ64_BALANCED = 7;        // products of a pass whose terms are balanced
 struct Oz64Geo {
   int Kh, rowsA, rowsB;
   CUtensorMap mapA, mapB;
@@ -67,7 +68,9 @@ struct Oz64 {
   void* base;
   char *SA, *SB;                        // slices of the left and the right operands
   int *eA, *eB;                         // row exponents
-  unsigned* mx;                         // row maxima (long rows)
+  int* mx;                              // exponents of the row maxima (long rows)
+  int* cm;                              // exponents of the terms' maxima, [product][item][2][kpitch]
+  int kpitch;
 };
 
 struct Plan {
@@ -179,7 +182,8 @@ cudaError_t after_launch(ntu_ctx* c, const char* name);
 // FP64 environment GEMMs on the tensor cores (k_oz64.cu)
 void oz64_init(ntu_ctx* c);
 void oz64_free(ntu_ctx* c);
-cudaError_t launch_oz64(ntu_ctx* c, const GemmOp& op, int gi, int n, const double2* A,
+cudaError_t oz64_begin(ntu_ctx* c);
+cudaError_t launch_oz64(ntu_ctx* c, const GemmOp& op, int gi, int slot, int n, const double2* A,
                         const double2* B, double2* C);
 
 // plans and tables (k_env.cu)
