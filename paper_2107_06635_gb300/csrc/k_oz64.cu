@@ -8,13 +8,20 @@
 // power of two into (-1, 1), rounded to 2^-54 and written as seven signed
 // digits of eight bits (|d| <= 128, exact in BF16):
 //   x = 2^(e-6) sum_i d_i 2^(-8 i),  i = 0 .. 6.
-// A product of two digits is an integer of at most 2^14, so the sums over up
-// to 256 terms of the at most four pairs (i, j) of one level l = i + j <= 3
-// stay below 2^24: their FP32 accumulators in tensor memory are exact.  Every
-// 256 terms they are drained into integer registers; levels 4 to 7, whose
-// rounding is below 2^-56 of the result's scale, accumulate over all terms,
-// and the levels above 7 (below 2^-64) are left out (without level 7 the sums
-// of 12 to 32 terms were up to 1.7 times less accurate than the FP64 chain).
+// A product of two digits is an integer of at most 2^14 (2^13 with a leading
+// digit, |d_0| <= 64), so the sums over up to 256 terms of the at most five
+// pairs (i, j) of one level l = i + j <= 4 stay within 2^24: their FP32
+// accumulators in tensor memory are exact.  Every 256 terms they are drained
+// into integer registers; levels 5 to 7 accumulate over all terms, and the
+// levels above 7 (below 2^-64) are left out (without level 7 the sums of 12 to
+// 32 terms were up to 1.7 times less accurate than the FP64 chain).  Those are
+// exact too up to 170 terms; beyond, digits of one sign (equal entries) can
+// bring level 5 to 2^16.4 a term, rounded to 24 bits at each of its 6 N / 16
+// accumulations: at the N = 8192 of the D = 8 join at most 2^17.6 units of
+// 2^-40, i.e. 2^-45 of a sum of equal terms.  With level 4 left to accumulate
+// as well the metric of equal entries was off by up to 2.7e-13 at D = 8, where
+// the FP64 chain is by 1.1e-13; now by 1.1e-14.  Digits without a pattern
+// stay exact at every level.
 // The epilogue joins the levels as integers and rounds once to FP64, without
 // FP64 instructions (one holds the pipe of a quarter of the SM for 64 cycles).
 // What is left is the operands' rounding to 2^-55 of their row's largest entry.
@@ -44,8 +51,8 @@
 // One persistent CTA per SM: warp 0 fetches stages of 32 real terms of all
 // seven slices (TMA boxes 32 x rows x 7, 64-byte swizzle), warp 1 issues the
 // MMAs (A slice i against B slices 0 .. 7-i, which are contiguous rows of
-// shared memory: accumulator columns 64 l .. hold level l; 11 instructions per
-// 16 terms), sixteen warps drain.  The 64 x 64 complex tile (all 512 TMEM
+// shared memory: accumulator columns 64 l .. hold level l; 13 instructions and
+// 34 digit products per 16 terms), sixteen warps drain.  The 64 x 64 complex tile (all 512 TMEM
 // columns) is single-buffered: the drain costs about a tenth of the products
 // of 256 terms.
 #include <cuda.h>
@@ -210,17 +217,20 @@ __global__ void __launch_bounds__(ZTHREADS, 1) k_oz64_gemm(const __grid_constant
             for (int i = 0; i < ZS; ++i) {
               const uint64_t ai = da + (uint64_t)(i * (ZA_SLICE >> 4) + 2 * kk);
               const uint64_t b0 = db + (uint64_t)(2 * kk);
-              if (i < 4)                                      // levels i .. 3
-                tc::mma_bf16(tmem + 64 * i, ai, b0, tc::idesc_bf16_f32(128, (4 - i) * 64),
-                             !(first && kk == 0 && i == 0));
-              // levels l0 .. 7 (there is no slice 7 for i = 0, and level 7 starts at i = 1)
-              const int l0 = i < 4 ? 4 : i, cut = i == 0 || (i == 1 && it == 0 && kk == 0) ? 7 : 8;
-              const uint64_t b4 = b0 + (uint64_t)((l0 - i) * (ZB_SLICE >> 4));
-              tc::mma_bf16(tmem + 64 * l0, ai, b4, tc::idesc_bf16_f32(128, (cut - l0) * 64),
-                           !(it == 0 && kk == 0 && i == 0));
-              if (i == 1 && cut == 7)
-                tc::mma_bf16(tmem + 64 * 7, ai, b0 + (uint64_t)(6 * (ZB_SLICE >> 4)),
-                             tc::idesc_bf16_f32(128, 64), 0);
+              // levels l .. l + n - 1: slices l - i .. of B
+              auto levels = [&](int l, int n, uint32_t add) {
+                tc::mma_bf16(tmem + 64 * l, ai, b0 + (uint64_t)((l - i) * (ZB_SLICE >> 4)),
+                             tc::idesc_bf16_f32(128, n * 64), add);
+              };
+              // the drained levels i .. 4 (256 columns at most), begun by i = 0
+              const uint32_t add = !(first && kk == 0 && i == 0);
+              if (i < 5) levels(i, i == 0 ? 4 : 5 - i, add);
+              if (i == 0) levels(4, 1, add);
+              // the levels to 7 (there is no slice 7 for i = 0: i = 1 begins level 7)
+              const int l0 = i < 5 ? 5 : i;
+              const bool split = i == 1 && it == 0 && kk == 0;
+              levels(l0, (i == 0 || split ? 7 : 8) - l0, !(it == 0 && kk == 0 && i == 0));
+              if (split) levels(7, 1, 0);
             }
           tc::mma_commit(&empty[s]);
           if (it % ZCHUNK == ZCHUNK - 1 || it == a.stages - 1) {
@@ -242,11 +252,10 @@ __global__ void __launch_bounds__(ZTHREADS, 1) k_oz64_gemm(const __grid_constant
     for (long long t = blockIdx.x; t < total && ok; t += gridDim.x) {
       const int z = (int)(t / per_item), rem = (int)(t % per_item);
       const int mt = rem / a.ntiles, nt = rem % a.ntiles;
-      int acc[4][16];
+      long long hi[16];                                      // levels 0 .. 3
+      int l4[16];
 #pragma unroll
-      for (int l = 0; l < 4; ++l)
-#pragma unroll
-        for (int q = 0; q < 16; ++q) acc[l][q] = 0;
+      for (int q = 0; q < 16; ++q) { hi[q] = 0; l4[q] = 0; }
       for (int it = 0; it < a.stages; it += ZCHUNK, ++chunk) {
         const bool got = tc::mbar_wait(accf, (uint32_t)(chunk & 1), ZWAIT);
         if (!tc::bar_and(1, ethreads, got)) {
@@ -255,13 +264,17 @@ __global__ void __launch_bounds__(ZTHREADS, 1) k_oz64_gemm(const __grid_constant
           break;
         }
         tc::fence_after_sync();
-#pragma unroll
+#pragma unroll 1
         for (int l = 0; l < 4; ++l) {
           float v[16];
           tc::tmem_ld16(tb + 64 * l, v);
 #pragma unroll
-          for (int q = 0; q < 16; ++q) acc[l][q] += __float2int_rn(v[q]);
+          for (int q = 0; q < 16; ++q) hi[q] += (long long)__float2int_rn(v[q]) << (24 - 8 * l);
         }
+        float v[16];
+        tc::tmem_ld16(tb + 64 * 4, v);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) l4[q] += __float2int_rn(v[q]);
         if (it + ZCHUNK < a.stages) {
           tc::fence_before_sync();
           __syncwarp();
@@ -269,17 +282,15 @@ __global__ void __launch_bounds__(ZTHREADS, 1) k_oz64_gemm(const __grid_constant
         }
       }
       if (!ok) break;
-      long long hi[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q)
-        hi[q] = ((((((long long)acc[0][q] << 8) + acc[1][q]) << 8) + acc[2][q]) << 8) + acc[3][q];
       long long lo[16];
 #pragma unroll
-      for (int l = 4; l < 8; ++l) {
+      for (int q = 0; q < 16; ++q) lo[q] = l4[q];
+#pragma unroll
+      for (int l = 5; l < 8; ++l) {
         float v[16];
         tc::tmem_ld16(tb + 64 * l, v);
 #pragma unroll
-        for (int q = 0; q < 16; ++q) lo[q] = (l > 4 ? lo[q] << 8 : 0) + __float2int_rn(v[q]);
+        for (int q = 0; q < 16; ++q) lo[q] = (lo[q] << 8) + __float2int_rn(v[q]);
       }
       tc::fence_before_sync();
       __syncwarp();
