@@ -418,11 +418,17 @@ __device__ __forceinline__ long long oz64_fix(double x, int em, int f) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   int ex = (int)(b >> 52) & 0x7ff;
   unsigned long long m = b & 0xfffffffffffffull;
-  if (ex) m |= 0x10000000000000ull;
-  else ex = 1;
-  const int sh = em - 1 - (ex + f);                       // >= -1, below for subnormals
-  const long long v = sh <= 0 ? (long long)(m << (-sh & 63))
-                              : (sh < 56 ? (long long)((m + (1ull << (sh - 1))) >> sh) : 0ll);
+  if (ex) {
+    m |= 0x10000000000000ull;
+  } else {                                                // subnormal (or 0, which stays 0)
+    const int z = __clzll((long long)m) - 11;
+    m <<= z;
+    ex = 1 - z;
+  }
+  const int sh = em - 1 - ex - f;                         // >= -1
+  const long long v = sh < 0 ? (long long)(m << 1)
+                             : (sh == 0 ? (long long)m
+                                        : (sh < 56 ? (long long)((m + (1ull << (sh - 1))) >> sh) : 0ll));
   return (long long)b < 0 ? -v : v;
 }
 
@@ -437,17 +443,22 @@ __global__ void __launch_bounds__(256) k_oz64_slice(Oz64Slice s) {
   {
     const int r = r0 + lane;
     int m = ZNONE;
+    const double2* p = s.src + z * s.s_src + (r < s.rows ? s.row[r] : 0);
+    double2 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = k0 + w + 8 * i;
+      v[i] = make_double2(0.0, 0.0);
+      if (r < s.rows && k < s.K) v[i] = p[s.kk[k]];
+    }
     if (threadIdx.x < 64) fac[threadIdx.x] = oz64_factor(s, z, k0 + (int)threadIdx.x);
     __syncthreads();
-    const double2* p = s.src + z * s.s_src + (r < s.rows ? s.row[r] : 0);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = w + 8 * i;
-      double2 v = make_double2(0.0, 0.0);
-      if (r < s.rows && k0 + k < s.K) v = p[s.kk[k0 + k]];
-      if (s.conj) v.y = -v.y;
-      tile[k * 33 + lane] = v;
-      m = max(m, oz64_exp(v) + fac[k]);
+      if (s.conj) v[i].y = -v[i].y;
+      tile[k * 33 + lane] = v[i];
+      m = max(m, oz64_exp(v[i]) + fac[k]);
     }
     red[w][lane] = m;
     __syncthreads();
