@@ -250,6 +250,7 @@ int ntu::init_context(const ntu_config* cfg, void* stream, ntu_ctx** out, int ma
     if (e == cudaSuccess) e = gate_qr_attributes();
     if (e == cudaSuccess) e = t12_attributes();
     if (e == cudaSuccess) e = tc_attributes();
+    if (e == cudaSuccess && f.precision == NTU_MIXED_FP32) e = cgemm32_attributes();
     if (e != cudaSuccess) {
       int st = cuda_check(nullptr, e, "device attributes");
       if (c->own_stream) cudaStreamDestroy(c->stream);

@@ -244,6 +244,22 @@ struct Cgemm32Tile { int tm, tn; Cgemm32 fn[2]; };          // fn[conjB]
 static const Cgemm32Tile c32_tiles[] = {C32(2, 2), C32(4, 2), C32(5, 2), C32(7, 2), C32(8, 2), C32(4, 4),
                                         C32(5, 4), C32(7, 4), C32(8, 4), C32(5, 7), C32(6, 5)};
 #undef C32
+static constexpr int c32_bytes(const Cgemm32Tile& t, int stages) {
+  return (int)sizeof(float2) * C32_BK * (8 * t.tm + 32 * t.tn) * stages;
+}
+
+// The limits belong to the functions, not to a context: every tile gets that of
+// its longest sums once, so that host threads (and captured graphs) never meet
+// another's.
+cudaError_t cgemm32_attributes() {
+  for (const Cgemm32Tile& t : c32_tiles)
+    for (Cgemm32 fn : t.fn) {
+      const cudaError_t e =
+          cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, c32_bytes(t, C32_STAGES));
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
+}
 
 // The tile with the least time by count: waves of two CTAs per SM times the
 // multiply-adds of a tile (rows and columns padded to it), times 1 + (shared
@@ -277,9 +293,7 @@ static cudaError_t run_gemm(ntu_ctx* c, const GemmOp& op, int n, const void* A, 
     const Cgemm32Tile& t32 = cgemm32_pick(op.M, op.N, n, c->sms);
     const Cgemm32 fn = t32.fn[op.conjB ? 1 : 0];
     const int bm = 8 * t32.tm, bn = 32 * t32.tn, chunks = (op.Kd + C32_BK - 1) / C32_BK;
-    const int smem = (int)sizeof(float2) * C32_BK * (bm + bn) * (chunks < C32_STAGES ? chunks : C32_STAGES);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
+    const int smem = c32_bytes(t32, chunks < C32_STAGES ? chunks : C32_STAGES);
     fn<<<dim3((op.N + bn - 1) / bn, (op.M + bm - 1) / bm, n), 256, smem, c->stream>>>(
         a, (const float2*)A, (const float2*)B, (float2*)C);
     return after_launch(c, "k_cgemm32");

@@ -496,8 +496,7 @@ static cudaError_t run_repair(ntu_ctx* c, int n, const C2in* graw, double2* g, d
   k_herm_certify<C2in><<<n, CERT_THREADS, 0, c->stream>>>(P.ng, graw, scale, trace, W.gscr, cert);
   e = after_launch(c, "k_herm_certify");
   if (e != cudaSuccess) return e;
-  const size_t sm = 2 * sizeof(double) * P.ng;
-  cudaFuncSetAttribute(k_repair<C2in>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  const size_t sm = 2 * sizeof(double) * P.ng;             // at most 16 KB: no limit to set
   k_repair<C2in><<<n, NTU_CTA, sm, c->stream>>>(P.ng, graw, g, W.gscr, W.gw, W.gz, W.geig, W.gtau,
                                                 W.gp, diag, c->d_status, c->d_paths, scale, cert);
   return after_launch(c, "k_repair");

@@ -225,10 +225,11 @@ size_t als_smem_bytes();
 long long oz_rows_side(int K);
 // Dynamic shared-memory limits of the fixed-size kernels, set on the
 // current device when a context is created there (k_gate_qr.cu, k_t12.cu,
-// k_tc.cu).
+// k_tc.cu; FP32 contexts: k_env.cu).
 cudaError_t gate_qr_attributes();
 cudaError_t t12_attributes();
 cudaError_t tc_attributes();
+cudaError_t cgemm32_attributes();
 
 // tensor-core environment (k_tc.cu, k_env.cu)
 int tc_make_map(CUtensorMap* map, void* base, long long cols, long long rows, long long items,
