@@ -335,18 +335,18 @@ __global__ void __launch_bounds__(NTU_CTA) k_qr(int m, int K, double2* __restric
   }
 }
 
-// The same factorisation on a cluster of CL CTAs, for the FP64 contexts with
-// few matrices: one SM's FP64 pipe took 0.94 ms at m = 1024, K = 16 (a
-// simple-update step at D = 8, with the recomposition and the estimator on
-// clusters too: 8.24 -> 4.25 ms).  Each CTA
-// holds a run of rows; the norm (each CTA's largest entry and its sum of
-// squares relative to that) and the inner products with the later columns go
-// to every CTA's shared memory and are added there in the order of the ranks,
-// so all CTAs go on with the same numbers: two cluster barriers a reflector, one
-// a column of Q.  Two buffers per exchange, by its number: a CTA can be one
-// barrier ahead of another's reads, never two.
+// The same factorisation, bit for bit, on a cluster of CL CTAs, for the FP64
+// contexts with few matrices: one SM's FP64 pipe took 0.94 ms at m = 1024, K = 16
+// (a simple-update step at D = 8, with the recomposition and the estimator on
+// clusters too: 8.24 -> 4.59 ms).  An item's result must not depend on how many
+// items go with it, so every sum keeps its order: column c belongs to CTA c % CL,
+// which forms its reflector (with k_qr's threads) and its inner products, the
+// real and the imaginary part on a warp each (two chains that never meet);
+// what has no order, the updates, is spread over the CTA.  One cluster barrier a
+// reflector (the column through global memory, its factors into every CTA's
+// shared memory), none for the columns of Q.
 constexpr int CL = 8;                                    // the portable cluster size
-struct QrHead { double mx, s2; double2 alpha; };         // a CTA's part of a column's norm
+static_assert(NTU_WARPS == 8 && CL == NTU_WARPS, "four columns of a CTA on eight warps; k_recompose");
 __global__ void __launch_bounds__(NTU_CTA) k_qr_cluster(int m, int K, double2* __restrict__ Mg,
                                                         double2* __restrict__ Qcm,
                                                         double2* __restrict__ QA, double2* __restrict__ RA,
@@ -355,10 +355,7 @@ __global__ void __launch_bounds__(NTU_CTA) k_qr_cluster(int m, int K, double2* _
   __shared__ double2 taus[32];
   __shared__ double betas[32];
   __shared__ double sred[2 * NTU_WARPS];
-  __shared__ QrHead head[2][CL];
-  __shared__ double2 dots[2][CL][32];
-  __shared__ double2 f[32];
-  __shared__ double sc[8];
+  __shared__ double dots[4][2];
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), item = blockIdx.x / CL, side = blockIdx.y, tid = threadIdx.x;
@@ -367,113 +364,64 @@ __global__ void __launch_bounds__(NTU_CTA) k_qr_cluster(int m, int K, double2* _
   cl.sync();                                             // every CTA is there to be written to
   double2* M = Mg + ((size_t)item * 2 + side) * m * K;
   double2* Qc = Qcm + ((size_t)item * 2 + side) * m * K;
-  const int run = (m + CL - 1) / CL, r0 = min(rank * run, m), r1 = min(r0 + run, m);
-  int ex = 0;                                            // number of the exchange of inner products
-  // f[c] = w sum conj(v) X[:, c] for columns c0 <= c < K, over all rows >= j
-  auto project = [&](const double2* v, const double2* X, int j, int c0, double2 w) {
-    for (int c = c0 + wid; c < K; c += NTU_WARPS) {
-      const double2* x = X + (size_t)c * m;
-      double2 dot = cz();
-      for (int i = max(r0, j) + lid; i < r1; i += 32) dot = cfmac(v[i], x[i], dot);
-      dot = warp_sum2(dot);
-      if (lid < CL) *cl.map_shared_rank(&dots[ex & 1][rank][c], lid) = dot;
+  // X[:, c] -= f v for the CTA's columns c >= c0, f = w v^H X[:, c], rows j ..
+  auto apply = [&](const double2* v, double2* X, int j, int c0, double2 w) {
+    const int first = c0 + ((rank - c0) & (CL - 1)), nc = first < K ? (K - 1 - first) / CL + 1 : 0;
+    if (nc == 0) return;                                 // the same in every thread
+    if (wid < 2 * nc) {
+      const double2* x = X + (size_t)(first + CL * (wid >> 1)) * m;
+      const bool im = wid & 1;
+      double dot = 0.0;
+      for (int i = j + lid; i < m; i += 32) {
+        const double2 a = v[i], b = x[i];
+        dot = fma(a.x, im ? b.y : b.x, dot);
+        dot = fma(a.y, im ? -b.x : b.y, dot);
+      }
+      dot = warp_sum(dot);
+      if (lid == 0) dots[wid >> 1][wid & 1] = dot;
     }
-    cl.sync();
-    if (tid >= c0 && tid < K) {
-      double2 t = dots[ex & 1][0][tid];
-      for (int q = 1; q < CL; ++q) t = cadd(t, dots[ex & 1][q][tid]);
-      f[tid] = cmul(w, t);
+    __syncthreads();
+    const int per = NTU_WARPS / nc, q = wid / per;       // warps of a column
+    if (q < nc) {
+      double2* x = X + (size_t)(first + CL * q) * m;
+      const double2 f = cmul(w, make_double2(dots[q][0], dots[q][1]));
+      for (int i = j + (wid % per) * 32 + lid; i < m; i += 32 * per) x[i] = cfms(f, v[i], x[i]);
     }
-    ++ex;
     __syncthreads();
   };
   for (int j = 0; j < K; ++j) {
     double2* col = M + (size_t)j * m;
-    const int i0 = max(r0, j + 1);
-    double mx = 0.0, xs2 = 0.0;
-    for (int i = i0 + tid; i < r1; i += NTU_CTA) mx = fmax(mx, fmax(fabs(col[i].x), fabs(col[i].y)));
-    mx = block_max(mx, sred);
-    if (mx > 0.0) {
-      const double inv = 1.0 / mx;
-      for (int i = i0 + tid; i < r1; i += NTU_CTA) xs2 += cabs2(cscale(col[i], inv));
-    }
-    xs2 = block_sum(xs2, sred);
-    if (tid < CL) {
-      const bool own = j >= r0 && j < r1;
-      const double2 al = own ? col[j] : cz();
-      *cl.map_shared_rank(&head[j & 1][rank], tid) = QrHead{mx, xs2, al};
+    if (j % CL == rank) {
+      const Reflector R = cta_reflector(col + j, m - j, sred);
+      __syncthreads();
+      for (int i = j + 1 + tid; i < m; i += NTU_CTA) col[i] = cmul(col[i], R.scale);
+      if (tid == 0) col[j] = make_double2(1.0, 0.0);
+      if (tid < CL) {
+        *cl.map_shared_rank(&taus[j], tid) = R.tau;
+        *cl.map_shared_rank(&betas[j], tid) = R.beta;
+      }
     }
     cl.sync();
-    if (tid == 0) {
-      double2 alpha = cz();
-      double big = 0.0, s2 = 0.0;
-      for (int q = 0; q < CL; ++q) {
-        const QrHead h = head[j & 1][q];
-        big = fmax(big, h.mx);
-        alpha = cadd(alpha, h.alpha);                    // one of them has the row
-      }
-      double2 tau = cz(), scale = make_double2(1.0, 0.0);
-      double beta = alpha.x;
-      if (!(big == 0.0 && alpha.y == 0.0)) {
-        const double amax = fmax(big, fmax(fabs(alpha.x), fabs(alpha.y))), inv = 1.0 / amax;
-        for (int q = 0; q < CL; ++q) {
-          const QrHead h = head[j & 1][q];
-          const double t = h.mx * inv;
-          if (h.mx > 0.0) s2 = fma(h.s2, t * t, s2);
-        }
-        const double nrm = amax * sqrt(cabs2(cscale(alpha, inv)) + s2);
-        beta = alpha.x >= 0.0 ? -nrm : nrm;
-        tau = make_double2((beta - alpha.x) / beta, -alpha.y / beta);
-        scale = cdiv(make_double2(1.0, 0.0), make_double2(alpha.x - beta, alpha.y));
-      }
-      taus[j] = tau;
-      betas[j] = beta;
-      sc[0] = scale.x;
-      sc[1] = scale.y;
-    }
-    __syncthreads();
-    const double2 tau = taus[j], scale = make_double2(sc[0], sc[1]);
-    for (int i = i0 + tid; i < r1; i += NTU_CTA) col[i] = cmul(col[i], scale);
-    if (tid == 0 && j >= r0 && j < r1) col[j] = make_double2(1.0, 0.0);
-    __syncthreads();
-    if ((tau.x != 0.0 || tau.y != 0.0) && j + 1 < K) {
-      project(col, M, j, j + 1, cconj(tau));
-      for (int c = j + 1 + wid; c < K; c += NTU_WARPS) {
-        double2* x = M + (size_t)c * m;
-        const double2 fc = f[c];
-        for (int i = max(r0, j) + lid; i < r1; i += 32) x[i] = cfms(fc, col[i], x[i]);
-      }
-      __syncthreads();
-    }
+    const double2 tau = taus[j];
+    if (tau.x != 0.0 || tau.y != 0.0) apply(col, M, j, j + 1, cconj(tau));
   }
   // Q = H_0 ... H_{K-1} [I; 0]
-  for (int c = wid; c < K; c += NTU_WARPS)
-    for (int i = r0 + lid; i < r1; i += 32) Qc[(size_t)c * m + i] = make_double2(i == c ? 1.0 : 0.0, 0.0);
+  for (int c = rank; c < K; c += CL)
+    for (int i = tid; i < m; i += NTU_CTA) Qc[(size_t)c * m + i] = make_double2(i == c ? 1.0 : 0.0, 0.0);
   __syncthreads();
   for (int j = K - 1; j >= 0; --j) {
     const double2 tau = taus[j];
-    if (tau.x == 0.0 && tau.y == 0.0) continue;
-    const double2* v = M + (size_t)j * m;
-    project(v, Qc, j, j, tau);
-    for (int c = j + wid; c < K; c += NTU_WARPS) {
-      double2* x = Qc + (size_t)c * m;
-      const double2 fc = f[c];
-      for (int i = max(r0, j) + lid; i < r1; i += 32) x[i] = cfms(fc, v[i], x[i]);
-    }
-    __syncthreads();
+    if (tau.x != 0.0 || tau.y != 0.0) apply(M + (size_t)j * m, Qc, j, j, tau);
   }
   double2* Qo = (side ? QB : QA) + (size_t)item * m * K;
   double2* Ro = (side ? RB : RA) + (size_t)item * K * K;
-  for (int idx = tid; idx < (r1 - r0) * K; idx += NTU_CTA) {
-    const int i = r0 + idx / K, c = idx % K;
-    const double2 q = Qc[(size_t)c * m + i];
-    Qo[(size_t)i * K + c] = betas[c] < 0.0 ? make_double2(-q.x, -q.y) : q;
-  }
-  const int k1 = min(r1, K);
-  for (int idx = tid; r0 < k1 && idx < (k1 - r0) * K; idx += NTU_CTA) {
-    const int j = r0 + idx / K, c = idx % K;
-    const double2 v = c > j ? M[(size_t)c * m + j] : (c == j ? make_double2(betas[j], 0.0) : cz());
-    Ro[j * K + c] = betas[j] < 0.0 ? make_double2(-v.x, -v.y) : v;
+  for (int c = rank; c < K; c += CL) {
+    const double sg = betas[c] < 0.0 ? -1.0 : 1.0;
+    for (int i = tid; i < m; i += NTU_CTA) Qo[(size_t)i * K + c] = cscale(Qc[(size_t)c * m + i], sg);
+    if (tid < K) {
+      const double2 v = c > tid ? M[(size_t)c * m + tid] : (c == tid ? make_double2(betas[tid], 0.0) : cz());
+      Ro[tid * K + c] = cscale(v, betas[tid] < 0.0 ? -1.0 : 1.0);
+    }
   }
 }
 
@@ -498,7 +446,9 @@ static cudaError_t launch_clusters(void (*kern)(P...), dim3 grid, cudaStream_t s
 // ------------------------------------------------------------ recompose
 // T' = Q M (Fig. 2(e)) put back into [p, l, u, r, dn] and normalised.
 // SPREAD: an item and side on a cluster (FP64 contexts with few items; 0.15 ms
-// on one SM at D = 8), the squared norm added over the CTAs.
+// on one SM at D = 8): CTA q takes the entries that the warp q of a single CTA
+// has, and its first warp adds their squares in that warp's order, so the norm
+// has the same bits.
 template <bool SPREAD>
 __global__ void __launch_bounds__(NTU_CTA) k_recompose(int dp, int D, int K,
                                                        const double2* __restrict__ QA,
@@ -512,8 +462,19 @@ __global__ void __launch_bounds__(NTU_CTA) k_recompose(int dp, int D, int K,
   __shared__ double sred[2 * NTU_WARPS];
   __shared__ double part[CL];
   const int item = SPREAD ? blockIdx.x / CL : blockIdx.x, side = blockIdx.y, tid = threadIdx.x;
-  const int rank = SPREAD ? blockIdx.x % CL : 0, step = SPREAD ? CL * NTU_CTA : NTU_CTA;
+  const int wid = tid >> 5, lid = tid & 31;
+  const int first = SPREAD ? wid * NTU_CTA + (blockIdx.x % CL) * 32 + lid : tid;
+  const int step = SPREAD ? NTU_WARPS * NTU_CTA : NTU_CTA;
   const int D2 = D * D, D3 = D2 * D, D4 = D3 * D, m = dp * D3;
+  // entry idx = row D + a of the product in [p, l, u, r, dn]
+  auto place = [&](int idx) {
+    const int row = idx / D, a = idx % D;
+    int n_ = row % D, t = row / D;
+    int u = t % D; t /= D;
+    int e = t % D; int p = t / D;
+    int l = side ? a : e, rr = side ? e : a;
+    return (size_t)p * D4 + l * D3 + u * D2 + rr * D + n_;
+  };
   const double2* Q = (side ? QB : QA) + (size_t)item * m * K;
   const double2* Mx = (side ? MB : MA) + (size_t)item * K * D;
   double2* out = (side ? TbO : TaO) + (size_t)item * dp * D4;
@@ -546,30 +507,39 @@ __global__ void __launch_bounds__(NTU_CTA) k_recompose(int dp, int D, int K,
         }
     }
   } else
-  for (int idx = rank * NTU_CTA + tid; idx < m * D; idx += step) {
-    int row = idx / D, a = idx % D;
+  for (int idx = first; idx < m * D; idx += step) {
+    const int row = idx / D, a = idx % D;
     double2 acc = cz();
     for (int k = 0; k < K; ++k) acc = cfma(Q[(size_t)row * K + k], Ms[k * D + a], acc);
-    int n_ = row % D, t = row / D;
-    int u = t % D; t /= D;
-    int e = t % D; int p = t / D;
-    int l = side ? a : e, rr = side ? e : a;
-    out[(size_t)p * D4 + l * D3 + u * D2 + rr * D + n_] = acc;
-    nrm2 += cabs2(acc);
+    out[place(idx)] = acc;
+    if (!SPREAD) nrm2 += cabs2(acc);
   }
-  nrm2 = block_sum(nrm2, sred);
   if (SPREAD) {
     cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
     cl.sync();                                           // every CTA is there to be written to
-    if (tid < CL) *cl.map_shared_rank(&part[rank], tid) = nrm2;
-    cl.sync();                                           // orders the CTAs' writes of out too
-    nrm2 = part[0];
-    for (int q = 1; q < CL; ++q) nrm2 += part[q];
+    if (wid == 0) {
+      for (int idx = first; idx < m * D; idx += NTU_CTA) nrm2 += cabs2(out[place(idx)]);
+      nrm2 = warp_sum(nrm2);
+      if (lid < CL) *cl.map_shared_rank(&part[blockIdx.x % CL], lid) = nrm2;
+    }
+    cl.sync();
+    nrm2 = 0.0;
+#pragma unroll
+    for (int q = 0; q < CL; ++q) nrm2 += part[q];
+  } else {
+    nrm2 = block_sum(nrm2, sred);
   }
   double nrm = sqrt(nrm2);
   double sc = nrm > 0.0 ? 1.0 / nrm : 1.0;
   __syncthreads();
-  for (int idx = rank * NTU_CTA + tid; idx < dp * D4; idx += step) out[idx] = cscale(out[idx], sc);
+  if (SPREAD) {
+    for (int idx = first; idx < m * D; idx += step) {
+      const size_t o = place(idx);
+      out[o] = cscale(out[o], sc);
+    }
+  } else {
+    for (int idx = tid; idx < dp * D4; idx += NTU_CTA) out[idx] = cscale(out[idx], sc);
+  }
 }
 
 // ------------------------------------------------------------ orientation
@@ -736,8 +706,8 @@ static inline int grid_for(long long work) {
 }
 
 // The FP64 contexts' QR and recomposition on clusters: where every item and side
-// has one at the same time, and there are rows to spread (16 a CTA: at m = 54, D = 3,
-// the whole QR takes one CTA 0.07 ms).
+// has one at the same time, and there are rows to spread (at m = 54, D = 3,
+// the whole QR takes one CTA 0.07 ms).  Same bits as on one CTA.
 static bool spread_items(const ntu_ctx* c, int n) {
   return c->cfg.precision == NTU_FP64 && (long long)n * 2 * CL <= c->sms && c->plan.m >= 128;
 }

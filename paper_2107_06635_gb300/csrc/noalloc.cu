@@ -7,7 +7,8 @@
 // (latency-critical loops sharing the GPU with other streams), or callers
 // that run where creating an ntu_ctx (which allocates its work space) is
 // not possible.  For them, ntu_gate_qr_noalloc runs the same three kernels
-// as an FP64 context's batch (k_gate_split, k_gated, k_qr), with their scratch --
+// as an FP64 context's batch (k_gate_split, k_gated, k_qr, whose bits the
+// clusters of a few items keep), with their scratch --
 // the split gate halves, the two gated site matrices and the Q work buffers
 // -- placed in one fixed, file-scope device array instead of the context's
 // work space.  The caller still passes inputs and outputs.
