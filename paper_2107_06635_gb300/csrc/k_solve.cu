@@ -182,8 +182,12 @@ __global__ void __launch_bounds__(256) k_herm_write(int ng, const C2in* __restri
 // that of the entries below 2^-24 tr H, so success proves H positive definite.
 // It decides metrics with lambda_min above some 1e-4 tr H at 64 times the FP64
 // rate (n = 400: 3.1 ms, bound by the trailing columns' traffic to L2, where the
-// FP64 Cholesky held the SM's FP64 pipe for 21 ms); a warp per column, four rows
-// a lane in flight.
+// FP64 Cholesky held the SM's FP64 pipe for 21 ms and the double-FP32 one 10 ms); a
+// warp per column, four rows a lane in flight.  A metric with a diagonal entry
+// below the shift cannot pass and is left alone: that is every graded one met
+// (of states part-way into a run); the attempt had made their repair in a mixed
+// context 3 to 13% longer (29.1 against 26.8 ms at n_g = 576).  A batch of both
+// kinds takes both, one after the other.
 // cert[item] = 1 where it succeeds; a block of CERT_THREADS per undecided item.
 constexpr int CERT_THREADS = 1024;
 template <typename C2in>
@@ -201,6 +205,9 @@ __global__ void __launch_bounds__(CERT_THREADS) k_herm_certify(int n, const C2in
   if (!(trace > 0x1p-900) || !(trace < 0x1p900)) return;
   const double f = scalbn(1.0, -ilogb(trace)), delta = 6.0 * (n + 3) * 0x1p-24 * trace;
   const C2in* gr = graw + item * (long long)n * n;
+  int low = 0;
+  for (int i = tid; i < n; i += CERT_THREADS) low |= !((double)gr[(size_t)i * n + i].x > delta);
+  if (__syncthreads_or(low)) return;
   float2* A = reinterpret_cast<float2*>(scr + item * (long long)n * n);
   for (int idx = tid; idx < n * n; idx += CERT_THREADS) {
     const int k = idx / n, i = idx % n;                     // column k, row i: conj of (k, i)

@@ -1,0 +1,48 @@
+"""Metrics that the Gershgorin discs leave open, with one diagonal entry next to
+the shift of the FP32 certificate (6 (n_g + 3) 2^-24 of the trace): definite ones
+are kept whichever factorisation proves it, indefinite ones clipped."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _metric(rng, n):
+    """Definite, eigenvalues in [0.5, 1.5], not diagonally dominant."""
+    w, _ = np.linalg.qr(rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n)))
+    g = (w * np.linspace(0.5, 1.5, n)) @ w.conj().T
+    return 0.5 * (g + g.conj().T)
+
+
+@pytest.mark.parametrize("D,r", [(4, 2), (6, 2), (4, 4), (5, 4)])
+def test_smallest_diagonal_next_to_the_shift(D, r):
+    import torch
+
+    from paper_2107_06635_gb300 import ntu
+
+    n = (D * r) ** 2
+    rng = np.random.default_rng(n)
+    shift = 6.0 * (n + 3) * 2.0 ** -24 * n
+    G = []
+    for i, f in enumerate((1e-9, 0.5, 0.99, 1.01, 2.0, 1e3)):
+        s = np.ones(n)
+        s[(7 * i) % n] = np.sqrt(f * shift)                  # a congruence: still definite
+        G.append(s[:, None] * _metric(rng, n) * s)
+    bad = _metric(rng, n)
+    bad[3, 3] = -0.2                                         # indefinite
+    G = np.stack([*G, bad])
+    g = torch.from_numpy(G).cuda()
+    diag = torch.empty((len(G), 3), dtype=torch.float64, device="cuda")
+    with ntu.Context(D, r=r, max_batch=len(G)) as ctx:
+        ctx.solver_paths()
+        ctx.batch_repair_dev(len(G), g, diag)
+        ctx.sync()
+        paths = ctx.solver_paths()
+    assert (paths["repair_gershgorin"], paths["repair_cholesky"], paths["repair_eigen"]) == (0, len(G) - 1, 1)
+    out = g.cpu().numpy()
+    for i in range(len(G) - 1):                              # scaled to unit trace, one rounding an entry
+        ref = G[i] / np.trace(G[i]).real
+        assert np.abs(out[i] - ref).max() <= n * 2.0 ** -52 * np.abs(ref).max()
+    lam, W = np.linalg.eigh(bad)
+    ref = (W * np.maximum(lam, 0)) @ W.conj().T
+    assert np.linalg.norm(out[-1] - ref / np.trace(ref).real) <= n * 2.0 ** -50 * np.linalg.norm(out[-1])
