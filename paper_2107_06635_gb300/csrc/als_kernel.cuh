@@ -784,18 +784,6 @@ static __device__ void als_source(AlsShared& sm, const AlsArgs& a, int side, dou
 // als_solve_spectrum (als_slow.cuh).
 static __device__ void als_mirror(double2* gX, int nA);
 
-// Upper triangle of the double-FP32 copy from its lower triangle.
-static __device__ void als_mirror_df(float4* A, int nA) {
-  for (int idx = threadIdx.x; idx < nA * nA; idx += NTU_CTA) {
-    const int col = idx / nA, row = idx % nA;
-    if (row < col) {
-      const float4 v = A[(size_t)row * nA + col];
-      A[idx] = make_float4(v.x, -v.y, v.z, -v.w);
-    }
-  }
-  __syncthreads();
-}
-
 // out = g_A v (g_A full, column-major), in FP64 or, with df, in double-FP32
 // on the copy scaled by 2^-ge (v is split into als_pdf(sm) first).  Two threads
 // per row take the two halves of the sum, each with two independent
@@ -890,6 +878,9 @@ static __device__ int als_solve_chol(AlsShared& sm, const AlsArgs& a, int side, 
   // reads every entry anyway (the product is dropped if tier 2 runs); that
   // rounding (< 1e-5 relative for n_A <= 256) is covered by inflating s_i by
   // 1e-4.
+  // (a.df is set in every launch of the mixed instances; left a run-time value,
+  // since without its branches the registers fall out worse: 45 updates at K = 32
+  // 32.0 against 30.2 ms)
   const bool df = !F64 && a.df != 0;
   const float4* gXdf = reinterpret_cast<const float4*>(gC);
   const double2* M0 = side == 0 ? sm.MA : sm.MB;

@@ -205,11 +205,12 @@ __device__ __forceinline__ double warp_max(double v) {
 
 // Sum over the CTA; every thread gets the result.  sbuf: >= NTU_WARPS*2 doubles.
 // LONE: thread 0 adds the warps' sums (in their order, so the same bits) where
-// otherwise every warp does.  Eight FP64 adds in eight warps take longer than in
-// one and a barrier more where a CTA has the SM to itself (the FP64 contexts:
-// 6.58 against 6.30 ms for a cell step at D = 3, with the tilts' roots in one warp),
-// not where three CTAs fill each other's waits (43.0 against 43.4 ms for 912
-// updates at D = 8).
+// otherwise every warp does: eight FP64 adds in eight warps against as many in
+// one and a barrier more.  It pays on the FP64 contexts, whose FP64 pipe is busy,
+// with one CTA on an SM (6.58 -> 6.30 ms for a cell step at D = 3, with the tilts'
+// roots in one warp) and with three (ALS of 912 updates at D = 3: 4.37 -> 3.33 ms;
+// of 456 at D = 4, r = 4: 21.3 -> 20.8), and costs on the mixed ones (43.0 against
+// 43.4 ms for 912 updates at D = 8).
 template <bool LONE = false>
 __device__ __forceinline__ double block_sum(double v, double* sbuf) {
   v = warp_sum(v);
@@ -891,49 +892,6 @@ __device__ inline int cta_cholesky_df(float4* __restrict__ A, int n, int* flag,
   int ok = *flag;
   __syncthreads();
   return ok;
-}
-
-// Solve (L L^H) x = b in place with the factor from cta_cholesky, by one
-// warp (no CTA barriers): lane l owns the entries i = l (mod 32) of b, which
-// lives in shared memory.  Must be called by all 32 lanes of one warp.
-__device__ inline void warp_cholesky_solve(const double2* __restrict__ L, int n, double2* b) {
-  const int lid = threadIdx.x & 31;
-  for (int j = 0; j < n; ++j) {           // L y = b
-    if ((j & 31) == lid) b[j] = cscale(b[j], 1.0 / L[(size_t)j * n + j].x);
-    __syncwarp();
-    const double2 yj = b[j];
-    const double2* cj = L + (size_t)j * n;
-    for (int i = j + 1 + ((lid - j - 1) & 31); i < n; i += 32) b[i] = cfms(cj[i], yj, b[i]);
-    __syncwarp();
-  }
-  for (int j = n - 1; j >= 0; --j) {      // L^H x = y
-    if ((j & 31) == lid) b[j] = cscale(b[j], 1.0 / L[(size_t)j * n + j].x);
-    __syncwarp();
-    const double2 xj = b[j];
-    for (int i = lid; i < j; i += 32) b[i] = cfmsc(xj, L[(size_t)i * n + j], b[i]);
-    __syncwarp();
-  }
-}
-
-// Solve (L L^H) x = b in place with the factor from cta_cholesky.
-__device__ inline void cta_cholesky_solve(const double2* __restrict__ L, int n, double2* b) {
-  const int tid = threadIdx.x;
-  for (int j = 0; j < n; ++j) {           // L y = b
-    __syncthreads();
-    double2 yj = cscale(b[j], 1.0 / L[(size_t)j * n + j].x);
-    __syncthreads();
-    if (tid == 0) b[j] = yj;
-    const double2* cj = L + (size_t)j * n;
-    for (int i = j + 1 + tid; i < n; i += NTU_CTA) b[i] = csub(b[i], cmul(cj[i], yj));
-  }
-  for (int j = n - 1; j >= 0; --j) {      // L^H x = y
-    __syncthreads();
-    double2 xj = cscale(b[j], 1.0 / L[(size_t)j * n + j].x);
-    __syncthreads();
-    if (tid == 0) b[j] = xj;
-    for (int i = tid; i < j; i += NTU_CTA) b[i] = csub(b[i], cmul(cconj(L[(size_t)i * n + j]), xj));
-  }
-  __syncthreads();
 }
 
 // u <- Z u (rotations replayed in reverse), single thread.
