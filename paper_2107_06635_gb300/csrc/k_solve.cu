@@ -175,6 +175,66 @@ __global__ void __launch_bounds__(256) k_herm_write(int ng, const C2in* __restri
   }
 }
 
+// The three in one, a block per item with a warp per row, for metrics whose
+// mirrored entries lie in L1: up to n_g = 64 the launches cost more than the
+// strided reads (n_g = 16, 48 metrics: 20 us a repair, 33 with three launches).
+constexpr int HERM_SMALL = 64;
+template <typename C2in>
+__global__ void __launch_bounds__(NTU_CTA) k_herm_small(int ng, const C2in* __restrict__ graw,
+                                                        double2* __restrict__ g, double* __restrict__ scale,
+                                                        double* __restrict__ trace, double* __restrict__ diag,
+                                                        int* paths) {
+  constexpr bool F32 = std::is_same<C2in, float2>::value;
+  typedef typename std::conditional<F32, float, double>::type R;
+  __shared__ double red[2 * NTU_WARPS], tw[NTU_WARPS];
+  const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
+  const long long item = blockIdx.x;
+  const C2in* gr = graw + item * (long long)ng * ng;
+  double2* gi = g + item * (long long)ng * ng;
+  R n2 = 0, h2 = 0;
+  double lo = INFINITY, t = 0.0;
+  for (int r = wid; r < ng; r += NTU_WARPS) {
+    R sr = 0;
+    double dr = 0.0;
+    for (int c = lid; c < ng; c += 32) {
+      const C2in a = gr[r * ng + c], b = gr[c * ng + r];
+      const R dx = a.x - b.x, dy = a.y + b.y;
+      n2 = fma(a.x, a.x, fma(a.y, a.y, n2));
+      h2 = fma(dx, dx, fma(dy, dy, h2));
+      if (c == r) dr = (double)a.x;
+      else sr += (R)0.5 * (fabs(a.x + b.x) + fabs(a.y - b.y));
+    }
+    const double d = warp_sum(dr);
+    const double s = F32 ? (double)warp_sum_f((float)sr) * (1.0 + 1e-4)
+                         : warp_sum((double)sr) * (1.0 + 1e-12);
+    lo = fmin(lo, d - s);
+    t += d;
+  }
+  lo = block_min(lo, red);
+  const double2 def = block_sum2(make_double2((double)n2, (double)h2), red);
+  if (lid == 0) tw[wid] = t;
+  __syncthreads();
+  double tr = 0.0;
+  for (int w = 0; w < NTU_WARPS; ++w) tr += tw[w];
+  const bool ok = lo > 0.0 && isfinite(lo) && tr > 0.0 && isfinite(tr);
+  const double hinv = 0.5 / tr;
+  if (ok)
+    for (int idx = tid; idx < ng * ng; idx += NTU_CTA) {
+      const double2 u = ld2(gr + idx), v = ld2(gr + (idx % ng) * ng + idx / ng);
+      gi[idx] = make_double2((u.x + v.x) * hinv, (u.y - v.y) * hinv);
+    }
+  if (tid == 0) {
+    scale[item] = ok ? hinv : 0.0;
+    trace[item] = tr;
+    diag[item * 3 + 0] = def.x > 0.0 ? sqrt(def.y / def.x) : 0.0;
+    if (ok) {
+      if (paths) atomicAdd(paths + 3, 1);
+      diag[item * 3 + 1] = __longlong_as_double(0x7ff8000000000000ULL);   // NaN
+      diag[item * 3 + 2] = log(tr);
+    }
+  }
+}
+
 // Whether H - delta I (H row-major, Hermitian) has an L D L^H
 // factorisation in FP32, delta = 6 (n + 3) 2^-24 tr H: the rounding of the
 // factorisation is a perturbation of at most 4 (n + 2) 2^-24 |L| |D| |L|^H,
@@ -286,7 +346,7 @@ __global__ void __launch_bounds__(NTU_CTA) k_repair(int ng, const C2in* __restri
   // (mixed contexts; it resolves it far below its own rounding), in FP64
   // otherwise
   constexpr bool kDf = std::is_same<C2in, float2>::value;
-  int ok = cert[item];
+  int ok = cert ? cert[item] : 0;
   if (!ok) {
     for (size_t idx = tid; idx < nn; idx += NTU_CTA) {      // column-major copy
       const size_t t = (idx % ng) * ng + idx / ng;
@@ -488,21 +548,32 @@ static cudaError_t run_repair(ntu_ctx* c, int n, const C2in* graw, double2* g, d
   RowStat* rows = reinterpret_cast<RowStat*>(W.gtau);       // n_g entries of 16 bytes per item
   double* scale = reinterpret_cast<double*>(W.x0);          // ALS scratch, free here
   double* trace = scale + n;
-  const int nb = (P.ng + 31) / 32;
-  k_herm_stats<C2in><<<dim3((unsigned)nb, (unsigned)n), 256, 0, c->stream>>>(P.ng, graw, rows, W.gp);
-  cudaError_t e = after_launch(c, "k_herm_stats");
-  if (e != cudaSuccess) return e;
-  k_herm_decide<<<n, NTU_CTA, 0, c->stream>>>(P.ng, rows, W.gp, scale, trace, diag, c->d_paths);
-  e = after_launch(c, "k_herm_decide");
-  if (e != cudaSuccess) return e;
-  k_herm_write<C2in><<<dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)n), 256, 0, c->stream>>>(
-      P.ng, graw, scale, g);
-  e = after_launch(c, "k_herm_write");
-  if (e != cudaSuccess) return e;
-  int* cert = reinterpret_cast<int*>(W.gx0);                // ALS scratch, free here
-  k_herm_certify<C2in><<<n, CERT_THREADS, 0, c->stream>>>(P.ng, graw, scale, trace, W.gscr, cert);
-  e = after_launch(c, "k_herm_certify");
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
+  if (P.ng <= HERM_SMALL) {
+    k_herm_small<C2in><<<n, NTU_CTA, 0, c->stream>>>(P.ng, graw, g, scale, trace, diag, c->d_paths);
+    e = after_launch(c, "k_herm_small");
+    if (e != cudaSuccess) return e;
+  } else {
+    const int nb = (P.ng + 31) / 32;
+    k_herm_stats<C2in><<<dim3((unsigned)nb, (unsigned)n), 256, 0, c->stream>>>(P.ng, graw, rows, W.gp);
+    e = after_launch(c, "k_herm_stats");
+    if (e != cudaSuccess) return e;
+    k_herm_decide<<<n, NTU_CTA, 0, c->stream>>>(P.ng, rows, W.gp, scale, trace, diag, c->d_paths);
+    e = after_launch(c, "k_herm_decide");
+    if (e != cudaSuccess) return e;
+    k_herm_write<C2in><<<dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)n), 256, 0, c->stream>>>(
+        P.ng, graw, scale, g);
+    e = after_launch(c, "k_herm_write");
+    if (e != cudaSuccess) return e;
+  }
+  // the FP32 certificate: from n_g = 33 on, below which the exact factorisation
+  // takes no longer than its launch
+  int* cert = P.ng > 32 ? reinterpret_cast<int*>(W.gx0) : nullptr;   // ALS scratch, free here
+  if (cert) {
+    k_herm_certify<C2in><<<n, CERT_THREADS, 0, c->stream>>>(P.ng, graw, scale, trace, W.gscr, cert);
+    e = after_launch(c, "k_herm_certify");
+    if (e != cudaSuccess) return e;
+  }
   const size_t sm = 2 * sizeof(double) * P.ng;             // at most 16 KB: no limit to set
   k_repair<C2in><<<n, NTU_CTA, sm, c->stream>>>(P.ng, graw, g, W.gscr, W.gw, W.gz, W.geig, W.gtau,
                                                 W.gp, diag, c->d_status, c->d_paths, scale, cert);

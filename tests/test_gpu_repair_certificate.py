@@ -46,3 +46,45 @@ def test_smallest_diagonal_next_to_the_shift(D, r):
     lam, W = np.linalg.eigh(bad)
     ref = (W * np.maximum(lam, 0)) @ W.conj().T
     assert np.linalg.norm(out[-1] - ref / np.trace(ref).real) <= n * 2.0 ** -50 * np.linalg.norm(out[-1])
+
+
+@pytest.mark.parametrize("D,r", [(1, 1), (2, 1), (2, 2), (5, 1), (3, 2), (7, 1), (4, 2), (3, 3), (6, 2)])
+def test_metrics_that_the_discs_decide(D, r):
+    """n_g = 1 to 144, on either side of the sizes that one block takes alone:
+    Hermitised, of unit trace, and the diagnostics; beside them one metric that
+    a factorisation decides and, from n_g = 4 on, one to be clipped."""
+    import torch
+
+    from paper_2107_06635_gb300 import ntu
+
+    n = (D * r) ** 2
+    rng = np.random.default_rng(10 * D + r)
+    noise = rng.standard_normal((3, n, n)) + 1j * rng.standard_normal((3, n, n))
+    G = [np.diag(rng.uniform(1, 2, n)) + x * (0.3 / (n + 1)) for x in noise]
+    if n > 1:
+        h = 0.5 * np.full((n, n), 1.9 / n) + np.eye(n)       # discs reach past zero from n = 21 on, definite
+        bad = np.eye(n) + 0j
+        bad[0, 1] = bad[1, 0] = 2.0                          # eigenvalue -1
+        G += [h + 0j, bad]
+    G = np.stack(G)
+    g = torch.from_numpy(G).cuda()
+    diag = torch.empty((len(G), 3), dtype=torch.float64, device="cuda")
+    with ntu.Context(D, r=r, max_batch=len(G)) as ctx:
+        ctx.solver_paths()
+        ctx.batch_repair_dev(len(G), g, diag)
+        ctx.sync()
+        paths = ctx.solver_paths()
+    assert paths["repair_eigen"] == (1 if n > 1 else 0)
+    assert paths["repair_gershgorin"] + paths["repair_cholesky"] == len(G) - paths["repair_eigen"]
+    assert paths["repair_gershgorin"] >= 3
+    out, diag = g.cpu().numpy(), diag.cpu().numpy()
+    for i, x in enumerate(G):
+        h = 0.5 * (x + x.conj().T)
+        defect = np.linalg.norm(x - x.conj().T) / np.linalg.norm(x)
+        assert abs(diag[i, 0] - defect) <= n * n * 2.0 ** -52 * max(defect, 1e-300)
+        lam, W = np.linalg.eigh(h)
+        ref = (W * np.maximum(lam, 0)) @ W.conj().T if i == 4 else h
+        tr = np.trace(ref).real
+        assert np.linalg.norm(out[i] - ref / tr) <= n * 2.0 ** -50 * np.linalg.norm(out[i])
+        assert abs(diag[i, 2] - np.log(tr)) <= n * 2.0 ** -50
+        assert np.isnan(diag[i, 1]) == (i != 4)
