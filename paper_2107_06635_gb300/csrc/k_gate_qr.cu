@@ -705,11 +705,18 @@ static inline int grid_for(long long work) {
   return (int)(b < 1 ? 1 : (b > 65535 ? 65535 : b));
 }
 
-// The FP64 contexts' QR and recomposition on clusters: where every item and side
-// has one at the same time, and there are rows to spread (at m = 54, D = 3,
-// the whole QR takes one CTA 0.07 ms).  Same bits as on one CTA.
+// The FP64 contexts' QR and recomposition on clusters (same bits as on one CTA):
+// where there are rows to spread (at m = 54, D = 3, the whole QR takes one CTA
+// 0.07 ms) and every CTA has an SM.  Clusters of eight do not fill the chip: up to
+// 3/4 of its SMs they stay apart (7 items: 0.53 against 0.99 ms at D = 8, r = 2;
+// 0.15 against 0.16 at D = 4), beyond some SMs hold two, which still pays for the
+// long columns (9 items: 0.63 ms at m K = 16384, 0.37 against 0.38 at 5184) and not
+// for the short ones (0.20 against 0.16 at 1024, 0.28 against 0.26 at 2500).
 static bool spread_items(const ntu_ctx* c, int n) {
-  return c->cfg.precision == NTU_FP64 && (long long)n * 2 * CL <= c->sms && c->plan.m >= 128;
+  const Plan& P = c->plan;
+  const long long ctas = (long long)n * 2 * CL;
+  return c->cfg.precision == NTU_FP64 && P.m >= 128 &&
+         (4 * ctas <= 3LL * c->sms || (ctas <= c->sms && P.m * P.K >= 5000));
 }
 
 cudaError_t launch_gate_qr(ntu_ctx* c, int n, const double2* Ta, const double2* Tb,
