@@ -41,6 +41,10 @@ __device__ __forceinline__ double2 ld2(const float2* p) {
 struct RowStat {
   double d, lo;                 // diagonal entry, disc's left end
 };
+// Shift of the FP32 certificate (k_herm_certify), and the multiple of it below
+// which a diagonal entry says that the attempt would hardly pass.
+__device__ __forceinline__ double cert_shift(int n, double tr) { return 6.0 * (n + 3) * 0x1p-24 * tr; }
+constexpr double CERT_DIAG = 3.0;
 
 template <typename C2in>
 __global__ void __launch_bounds__(256) k_herm_stats(int ng, const C2in* __restrict__ graw,
@@ -96,14 +100,19 @@ __global__ void __launch_bounds__(NTU_CTA) k_herm_decide(int ng, const RowStat* 
                                                          const double2* __restrict__ part,
                                                          double* __restrict__ scale,
                                                          double* __restrict__ trace,
-                                                         double* __restrict__ diag, int* paths) {
+                                                         double* __restrict__ diag, int* __restrict__ cert,
+                                                         int* paths) {
   __shared__ double red[2 * NTU_WARPS], tw[NTU_WARPS];
   const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
   const long long item = blockIdx.x;
   const RowStat* rs = rows + item * ng;
-  double lo = INFINITY;
-  for (int r = tid; r < ng; r += NTU_CTA) lo = fmin(lo, rs[r].lo);
+  double lo = INFINITY, dmin = INFINITY;
+  for (int r = tid; r < ng; r += NTU_CTA) {
+    lo = fmin(lo, rs[r].lo);
+    dmin = fmin(dmin, rs[r].d);
+  }
   lo = block_min(lo, red);
+  dmin = block_min(dmin, red);
   if (lid == 0) {
     double t = 0.0;
     for (int r = wid; r < ng; r += NTU_WARPS) t += rs[r].d;
@@ -117,6 +126,7 @@ __global__ void __launch_bounds__(NTU_CTA) k_herm_decide(int ng, const RowStat* 
     const bool ok = lo > 0.0 && isfinite(lo) && tr > 0.0 && isfinite(tr);
     scale[item] = ok ? 0.5 / tr : 0.0;
     trace[item] = tr;
+    cert[item] = ok || dmin > CERT_DIAG * cert_shift(ng, tr) ? 0 : -1;
     diag[item * 3 + 0] = n2 > 0.0 ? sqrt(h2 / n2) : 0.0;
     if (ok) {
       if (paths) atomicAdd(paths + 3, 1);
@@ -183,7 +193,7 @@ template <typename C2in>
 __global__ void __launch_bounds__(NTU_CTA) k_herm_small(int ng, const C2in* __restrict__ graw,
                                                         double2* __restrict__ g, double* __restrict__ scale,
                                                         double* __restrict__ trace, double* __restrict__ diag,
-                                                        int* paths) {
+                                                        int* __restrict__ cert, int* paths) {
   constexpr bool F32 = std::is_same<C2in, float2>::value;
   typedef typename std::conditional<F32, float, double>::type R;
   __shared__ double red[2 * NTU_WARPS], tw[NTU_WARPS];
@@ -192,7 +202,7 @@ __global__ void __launch_bounds__(NTU_CTA) k_herm_small(int ng, const C2in* __re
   const C2in* gr = graw + item * (long long)ng * ng;
   double2* gi = g + item * (long long)ng * ng;
   R n2 = 0, h2 = 0;
-  double lo = INFINITY, t = 0.0;
+  double lo = INFINITY, dmin = INFINITY, t = 0.0;
   for (int r = wid; r < ng; r += NTU_WARPS) {
     R sr = 0;
     double dr = 0.0;
@@ -208,9 +218,11 @@ __global__ void __launch_bounds__(NTU_CTA) k_herm_small(int ng, const C2in* __re
     const double s = F32 ? (double)warp_sum_f((float)sr) * (1.0 + 1e-4)
                          : warp_sum((double)sr) * (1.0 + 1e-12);
     lo = fmin(lo, d - s);
+    dmin = fmin(dmin, d);
     t += d;
   }
   lo = block_min(lo, red);
+  dmin = block_min(dmin, red);
   const double2 def = block_sum2(make_double2((double)n2, (double)h2), red);
   if (lid == 0) tw[wid] = t;
   __syncthreads();
@@ -226,6 +238,7 @@ __global__ void __launch_bounds__(NTU_CTA) k_herm_small(int ng, const C2in* __re
   if (tid == 0) {
     scale[item] = ok ? hinv : 0.0;
     trace[item] = tr;
+    cert[item] = ok || dmin > CERT_DIAG * cert_shift(ng, tr) ? 0 : -1;
     diag[item * 3 + 0] = def.x > 0.0 ? sqrt(def.y / def.x) : 0.0;
     if (ok) {
       if (paths) atomicAdd(paths + 3, 1);
@@ -244,30 +257,29 @@ __global__ void __launch_bounds__(NTU_CTA) k_herm_small(int ng, const C2in* __re
 // rate (n = 400: 3.1 ms, bound by the trailing columns' traffic to L2, where the
 // FP64 Cholesky held the SM's FP64 pipe for 21 ms and the double-FP32 one 10 ms); a
 // warp per column, four rows a lane in flight.  A metric with a diagonal entry
-// below the shift cannot pass and is left alone: that is every graded one met
-// (of states part-way into a run); the attempt had made their repair in a mixed
-// context 3 to 13% longer (29.1 against 26.8 ms at n_g = 576).  A batch of both
-// kinds takes both, one after the other.
-// cert[item] = 1 where it succeeds; a block of CERT_THREADS per undecided item.
+// below the shift cannot pass, and one below three times it hardly does: such a
+// metric (of a state part-way into a run, graded) is left alone, and where all
+// items run at once (n <= lone) so is the whole batch, which lasts as long as its
+// longest item: there the attempt had made the repair up to 31% longer (24 items at
+// D = 6: 1.12 ms, 0.87 now; one at D = 2, r = 16: 150, 124).
+// cert[item] = 1 where it succeeds (0 before; -1: left alone); a block of
+// CERT_THREADS per item.
 constexpr int CERT_THREADS = 1024;
 template <typename C2in>
 __global__ void __launch_bounds__(CERT_THREADS) k_herm_certify(int n, const C2in* __restrict__ graw,
                                                                const double* __restrict__ scale,
                                                                const double* __restrict__ traces,
-                                                               double2* __restrict__ scr,
+                                                               double2* __restrict__ scr, int lone,
                                                                int* __restrict__ cert) {
   __shared__ float2 col[1024];                              // n_g <= 1024
   const long long item = blockIdx.x;
   const int tid = threadIdx.x, wid = tid >> 5, lid = tid & 31;
-  if (tid == 0) cert[item] = 0;
-  if (scale[item] != 0.0) return;                           // decided by the discs
+  if (scale[item] != 0.0 || cert[item] < 0) return;         // decided by the discs; left alone
+  if ((int)gridDim.x <= lone && __syncthreads_or(tid < (int)gridDim.x && cert[tid] < 0)) return;
   const double trace = traces[item];
   if (!(trace > 0x1p-900) || !(trace < 0x1p900)) return;
-  const double f = scalbn(1.0, -ilogb(trace)), delta = 6.0 * (n + 3) * 0x1p-24 * trace;
+  const double f = scalbn(1.0, -ilogb(trace)), delta = cert_shift(n, trace);
   const C2in* gr = graw + item * (long long)n * n;
-  int low = 0;
-  for (int i = tid; i < n; i += CERT_THREADS) low |= !((double)gr[(size_t)i * n + i].x > delta);
-  if (__syncthreads_or(low)) return;
   float2* A = reinterpret_cast<float2*>(scr + item * (long long)n * n);
   for (int idx = tid; idx < n * n; idx += CERT_THREADS) {
     const int k = idx / n, i = idx % n;                     // column k, row i: conj of (k, i)
@@ -346,7 +358,7 @@ __global__ void __launch_bounds__(NTU_CTA) k_repair(int ng, const C2in* __restri
   // (mixed contexts; it resolves it far below its own rounding), in FP64
   // otherwise
   constexpr bool kDf = std::is_same<C2in, float2>::value;
-  int ok = cert ? cert[item] : 0;
+  int ok = cert[item] > 0;
   if (!ok) {
     for (size_t idx = tid; idx < nn; idx += NTU_CTA) {      // column-major copy
       const size_t t = (idx % ng) * ng + idx / ng;
@@ -548,9 +560,11 @@ static cudaError_t run_repair(ntu_ctx* c, int n, const C2in* graw, double2* g, d
   RowStat* rows = reinterpret_cast<RowStat*>(W.gtau);       // n_g entries of 16 bytes per item
   double* scale = reinterpret_cast<double*>(W.x0);          // ALS scratch, free here
   double* trace = scale + n;
+  int* cert = reinterpret_cast<int*>(W.gx0);                // ALS scratch, free here
   cudaError_t e;
   if (P.ng <= HERM_SMALL) {
-    k_herm_small<C2in><<<n, NTU_CTA, 0, c->stream>>>(P.ng, graw, g, scale, trace, diag, c->d_paths);
+    k_herm_small<C2in><<<n, NTU_CTA, 0, c->stream>>>(P.ng, graw, g, scale, trace, diag, cert,
+                                                          c->d_paths);
     e = after_launch(c, "k_herm_small");
     if (e != cudaSuccess) return e;
   } else {
@@ -558,7 +572,7 @@ static cudaError_t run_repair(ntu_ctx* c, int n, const C2in* graw, double2* g, d
     k_herm_stats<C2in><<<dim3((unsigned)nb, (unsigned)n), 256, 0, c->stream>>>(P.ng, graw, rows, W.gp);
     e = after_launch(c, "k_herm_stats");
     if (e != cudaSuccess) return e;
-    k_herm_decide<<<n, NTU_CTA, 0, c->stream>>>(P.ng, rows, W.gp, scale, trace, diag, c->d_paths);
+    k_herm_decide<<<n, NTU_CTA, 0, c->stream>>>(P.ng, rows, W.gp, scale, trace, diag, cert, c->d_paths);
     e = after_launch(c, "k_herm_decide");
     if (e != cudaSuccess) return e;
     k_herm_write<C2in><<<dim3((unsigned)(nb * (nb + 1) / 2), (unsigned)n), 256, 0, c->stream>>>(
@@ -568,9 +582,9 @@ static cudaError_t run_repair(ntu_ctx* c, int n, const C2in* graw, double2* g, d
   }
   // the FP32 certificate: from n_g = 33 on, below which the exact factorisation
   // takes no longer than its launch
-  int* cert = P.ng > 32 ? reinterpret_cast<int*>(W.gx0) : nullptr;   // ALS scratch, free here
-  if (cert) {
-    k_herm_certify<C2in><<<n, CERT_THREADS, 0, c->stream>>>(P.ng, graw, scale, trace, W.gscr, cert);
+  if (P.ng > 32) {
+    const int lone = c->sms < CERT_THREADS ? c->sms : CERT_THREADS;
+    k_herm_certify<C2in><<<n, CERT_THREADS, 0, c->stream>>>(P.ng, graw, scale, trace, W.gscr, lone, cert);
     e = after_launch(c, "k_herm_certify");
     if (e != cudaSuccess) return e;
   }

@@ -88,3 +88,38 @@ def test_metrics_that_the_discs_decide(D, r):
         assert np.linalg.norm(out[i] - ref / tr) <= n * 2.0 ** -50 * np.linalg.norm(out[i])
         assert abs(diag[i, 2] - np.log(tr)) <= n * 2.0 ** -50
         assert np.isnan(diag[i, 1]) == (i != 4)
+
+
+@pytest.mark.parametrize("D,r", [(3, 2), (6, 2)])
+@pytest.mark.parametrize("n", [4, 170])
+def test_result_does_not_depend_on_the_batch(D, r, n):
+    """Flat and graded metrics in one batch (below and above the number of items
+    that run at once, which decides whether the certificate is tried): every
+    result has the bits it has alone."""
+    import torch
+
+    from paper_2107_06635_gb300 import ntu
+
+    m = (D * r) ** 2
+    rng = np.random.default_rng(m)
+    shift = 6.0 * (m + 3) * 2.0 ** -24 * m
+    kinds = []
+    for f in (1e-6, 2.9, 3.1, 1e3):
+        s = np.ones(m)
+        s[1] = np.sqrt(f * shift)
+        kinds.append(s[:, None] * _metric(rng, m) * s)
+    which = np.arange(n) % 4
+
+    def repair(x):
+        g = torch.from_numpy(np.ascontiguousarray(x)).cuda()
+        diag = torch.empty((len(x), 3), dtype=torch.float64, device="cuda")
+        with ntu.Context(D, r=r, max_batch=len(x)) as ctx:
+            ctx.batch_repair_dev(len(x), g, diag)
+            ctx.sync()
+            assert ctx.solver_paths()["repair_cholesky"] == len(x)
+        return g.cpu().numpy()
+
+    alone = [repair(k[None])[0] for k in kinds]
+    out = repair(np.stack([kinds[w] for w in which]))
+    for i in range(n):
+        assert np.array_equal(out[i], alone[which[i]])
