@@ -62,7 +62,9 @@ typedef enum {
 } ntu_status;
 
 typedef enum {
-  NTU_FP64 = 0,          /* every step in FP64                                */
+  NTU_FP64 = 0,          /* every step in FP64; the long products of the      */
+                         /* environment from slices on the tensor cores,      */
+                         /* summed exactly and rounded once                   */
   NTU_MIXED_FP32 = 1,    /* environment contraction (Fig. 4) in FP32,         */
                          /* solvers in FP64                                   */
   NTU_MIXED_BF16X3 = 2   /* environment contraction with split-BF16 tensor-  */
@@ -101,7 +103,15 @@ typedef struct {
  * On the mixed contexts a max_batch of at most 3 * SMs / 2 (228 on 152 SMs)
  * lets each item's ALS run on a cluster of 2 CTAs, at most 3 * SMs / 4 on
  * 4 (same results, bit for bit); its ALS scratch is then allocated that many
- * times. */
+ * times.
+ * An FP64 context also takes scratch for the slices of its environment: what
+ * max_batch items need (90 MB an item at D = 8, r = 2, 350 MB at r = 4), at
+ * most 2 GB or one item's.  This one allocation may fail without an error (and
+ * is not made on a GPU without tcgen05): the environment then runs on the FP64
+ * pipe, with FP64's rounding instead of the slices' and up to 15 times slower.
+ * Contexts of an FP64 ntu_uneven take it for each kind.
+ * An item's result on one context does not depend on the other items of the
+ * call or on their number. */
 int ntu_init(const ntu_config* cfg, void* stream, ntu_ctx** out);
 int ntu_destroy(ntu_ctx* ctx);
 /* The last error message of `ctx`; with ctx == NULL, of the calling thread's
@@ -332,7 +342,7 @@ int ntu_uneven_get_tuning(const ntu_uneven* uneven, int kind, ntu_tuning* t, int
 
 /* CUDA graphs of the unit-cell step.  With graphs on (the default), the
  * device work of ntu_step and ntu_su_step -- the single-site gates and the
- * four bond updates, some 90 launches -- is captured as one CUDA graph on
+ * four bond updates, 90 to 230 launches -- is captured as one CUDA graph on
  * the first call (one graph per call form: with or without gate1_half) and
  * replayed by later calls; the gates are copied in before the replay and
  * the deltas read back after it.  Off: the same launches are issued one by

@@ -32,16 +32,16 @@
 // 2^((b_k - a_k) / 2) and the right one divided by it, in the exponents alone.
 // (Scales 1 .. 1e-8 on a leg and their inverses on its partner cost the metric
 // all its digits without.)  The edges are Gram products: a_k = b_k.
-// With that,
-// relative to 113-bit sums the metric at D = 2 to 4 is off by 1e-16 to 1e-15
-// where the FP64 chain was off by 3e-16 to 2.3e-15.
+// With that, relative to 113-bit sums the metric at D = 2 to 4 is off by 1e-16 to
+// 1e-15 where the FP64 chain was off by 3e-16 to 2.3e-15, of its norm; an entry far
+// below the norm keeps less relative accuracy than the chain gave it.
 //
-// Measured, environment of 48 bond updates at D = 8, r = 2: 13.3 ms against
-// 196.6 ms on the FP64 pipe; of one at D = 3: 0.44 against 1.2 ms (a 64 x 64
+// Measured, environment of 48 bond updates at D = 8, r = 2: 14.2 ms against
+// 196.6 ms on the FP64 pipe; of one at D = 3: 0.50 against 1.2 ms (a 64 x 64
 // FP64 tile of the SIMT product holds one SM for 0.3 ms whatever its padding),
-// so the sliced products run at every size.  Of the 13.3 ms the GEMMs take 8
+// so the sliced products run at every size.  Of the 14.2 ms the GEMMs take 7.4
 // (the join at 40% of the BF16 peak, t1 to h bound by their epilogues), the
-// slicing 5.
+// slices 3.5, the exponents of rows and terms 1.4, the side edges and Y 1.4.
 //
 // Complex products are one real GEMM: rows of B hold [Re | Im] along K, a
 // complex row of A the two real rows [Re | -Im] and [Im | Re].  They lie 16
